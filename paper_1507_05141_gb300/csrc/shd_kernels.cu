@@ -577,8 +577,9 @@ __device__ inline float fast_recip<float>(float x) { return hw_rcp(x); }
 // only for the 4-node pieces of a plane that hold a moving node (bit id % 64
 // of mbits[d][id / 64][piece]) and from chi0L elsewhere; the CTA keeps the
 // current 64-plane window of its layout's bits in shared memory.
-// WIDE: the transfer weights switch to FP64 above optical depth kFp64Tau
-// (launched unless the host bound excludes such steps).
+// WIDE (single precision): the weights' exponential carries the remainder of
+// its argument (exp_neg); launched unless the host bound excludes optical
+// depths above kTauPlain.
 template <class T, int U, bool VEC, bool CB, bool WIDE>
 __global__ void __launch_bounds__(1024, 1) k_sweep_pipe(Prob<T> P, T *__restrict__ I, const T *__restrict__ eta,
                                                         const T *__restrict__ chi, const T *__restrict__ chi0L,
@@ -1150,7 +1151,7 @@ __device__ inline T clamp_between(T v, T a, T b)
     return v < lo ? lo : (v > hi ? hi : v);
 }
 
-template <class T, int U, bool WIDE>
+template <class T, int U>
 __global__ void __launch_bounds__(1024, 1) k_sweep_bez(Prob<T> P, T *__restrict__ I, const T *__restrict__ eta,
                                                        const T *__restrict__ chi, int pstride)
 {
@@ -1194,7 +1195,7 @@ __global__ void __launch_bounds__(1024, 1) k_sweep_bez(Prob<T> P, T *__restrict_
             if (j >= plane) break;
             const T ct = Ch[u] + kap;
             Pair2<T> v;
-            v.x = ct > T(0) ? (Et[u] + kap * In[u]) / ct : T(0);
+            v.x = ct > T(0) ? (Et[u] + kap * In[u]) * recip<T>(ct) : T(0);
             v.y = ct;
             dst[j] = v;
         }
@@ -1248,7 +1249,7 @@ __global__ void __launch_bounds__(1024, 1) k_sweep_bez(Prob<T> P, T *__restrict_
                 if (p == 0 || ((fin >> u) & 1u)) {
                     inew = bc_full ? P.bc[pb + j] : bc_iso;
                     // the downwind slope; no derivative (NaN) without a downwind point
-                    dP = has_d ? (xd > T(0) ? (sD - sP) / xd : T(0)) : T(NAN);
+                    dP = has_d ? (xd > T(0) ? (sD - sP) * recip<T>(xd) : T(0)) : T(NAN);
                 } else {
                     const Quad4<T> q00 = up[j], q10 = up[j - d1], q01 = up[j - d2], q11 = up[j - d1 - d2];
                     const T iu = w00 * q00.x + w10 * q10.x + w01 * q01.x + w11 * q11.x;
@@ -1261,20 +1262,17 @@ __global__ void __launch_bounds__(1024, 1) k_sweep_bez(Prob<T> P, T *__restrict_
                     if (!isnan(q01.w)) { dsum += w01 * q01.w; dw += w01; }
                     if (!isnan(q11.w)) { dsum += w11 * q11.w; dw += w11; }
                     const T x = s * T(0.5) * (cu + cP);
-                    const T slope = x > T(0) ? (sP - su) / x : T(0);
-                    const T du = dw > T(0) ? dsum / dw : slope;
+                    const T rx = recip<T>(x);
+                    const T slope = x > T(0) ? (sP - su) * rx : T(0);
+                    const T du = dw > T(0) ? dsum * recip<T>(dw) : slope;
                     dP = slope;
-                    if (has_d) dP = (x > T(0) && xd > T(0)) ? fb_derivative<T>(slope, (sD - sP) / xd, x, xd) : T(0);
-                    const T Cu = clamp_between<T>(su + x * du / T(3), su, sP);
-                    const T Cp = clamp_between<T>(sP - x * dP / T(3), su, sP);
+                    if (has_d)
+                        dP = (x > T(0) && xd > T(0)) ? fb_derivative<T>(slope, (sD - sP) * recip<T>(xd), x, xd) : T(0);
+                    const T x3 = x * T(1.0 / 3.0);
+                    const T Cu = clamp_between<T>(su + x3 * du, su, sP);
+                    const T Cp = clamp_between<T>(sP - x3 * dP, su, sP);
                     T e, wU, wCU, wCP, wP;
-                    if (WIDE && sizeof(T) == 4 && x > T(kFp64Tau)) {
-                        double ed, a1, a2, a3, a4;
-                        bezier_weights<double>((double)x, ed, a1, a2, a3, a4);
-                        e = (T)ed; wU = (T)a1; wCU = (T)a2; wCP = (T)a3; wP = (T)a4;
-                    } else {
-                        bezier_weights<T>(x, e, wU, wCU, wCP, wP);
-                    }
+                    bezier_weights<T>(x, rx, e, wU, wCU, wCP, wP);
                     inew = iu * e + wU * su + wCU * Cu + wCP * Cp + wP * sP;
                 }
                 Quad4<T> v;
@@ -2065,13 +2063,13 @@ static cudaError_t launch_sweep_npt(const shd_ctx *ctx, T *I, const T *eta, cons
 
 // Optical depth of one short-characteristic step is at most s_max chi~_max
 // with chi~ = chi_lab + kappa and chi_lab <= chi0_max D_max, D = Gamma - u.n <
-// 2 Gamma (R17): true when that stays within kFp64Tau.
+// 2 Gamma (R17): true when that stays within kTauPlain.
 static bool sweep_tau_bounded(const shd_ctx *c)
 {
     double smax = 0;
     for (const Ordinate &o : c->h_ord) smax = o.s > smax ? o.s : smax;
     const double chi = (c->h_alpha_max + c->h_ne_max * c->h_sigma_max) * 2.0 * c->h_gamma_max + c->kappa;
-    return std::isfinite(chi) && smax * chi <= (double)kFp64Tau;
+    return std::isfinite(chi) && smax * chi <= (double)kTauPlain;
 }
 
 template <class T, int U, bool VEC>
@@ -2082,7 +2080,7 @@ static cudaError_t launch_sweep_pipe(const shd_ctx *ctx, T *I, const T *eta, con
     const T *c0L = bits ? (const T *)ctx->d_chi0L : nullptr;
     const unsigned long long *mb = bits ? ctx->d_mbits : nullptr;
     if (bits) sm += sizeof(unsigned long long) * (size_t)ctx->mbits_npc;
-    // FP64 weights are needed only if a step's optical depth can exceed kFp64Tau
+    // the compensated exponential is needed only if a step's optical depth can exceed kTauPlain
     const bool wide = sizeof(T) == 4 && !sweep_tau_bounded(ctx);
     auto kern = bits ? (wide ? k_sweep_pipe<T, U, VEC, VEC, (sizeof(T) == 4)> : k_sweep_pipe<T, U, VEC, VEC, false>)
                      : (wide ? k_sweep_pipe<T, U, VEC, false, (sizeof(T) == 4)> : k_sweep_pipe<T, U, VEC, false, false>);
@@ -2390,7 +2388,7 @@ int sweep_batch_class(const shd_ctx *c)
         }
         if (!(pp > 0.f && pp <= 1.03f * best)) return 0;
     }
-    // class: U (bits 0-2), chi0 table (bit 3), FP64 weights (bit 4)
+    // class: U (bits 0-2), chi0 table (bit 3), compensated exponential (bit 4)
     return sc.U | (sweep_uses_chi0L<float>(c) ? 8 : 0) | (sweep_tau_bounded(c) ? 0 : 16);
 }
 
@@ -2452,8 +2450,7 @@ static cudaError_t launch_sweep_bez_u(const shd_ctx *ctx, T *I, const T *eta, co
     Prob<T> P = make_prob<T>(ctx);
     const size_t sm = sweep_bez_smem_bytes(ctx);
     const int pstride = (int)(((size_t)sweep_plane_max(ctx) + 3) & ~(size_t)3);
-    const bool wide = sizeof(T) == 4 && !sweep_tau_bounded(ctx);
-    auto kern = wide ? k_sweep_bez<T, U, (sizeof(T) == 4)> : k_sweep_bez<T, U, false>;
+    auto kern = k_sweep_bez<T, U>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)(ctx->N * ctx->G), 1024, sm, st>>>(P, I, eta, chi, pstride);
