@@ -276,8 +276,8 @@ int shd_get_state_dev(shd_ctx *ctx, double *dev_I, void *cuda_stream);
  * most 4 NT nodes, several CTAs an SM; any grid) or split over a
  * thread-block cluster of C CTAs (C = 2, 4, 8 or 16; NT = 256, 384, 512, 768 or
  * 1024; grids whose planes and node count are multiples of 4), each CTA
- * owning a block of rows; rows next to another CTA's block read it through
- * distributed shared memory.  The result does not depend on the schedule
+ * owning a block of rows and receiving the row upwind of them from the
+ * neighbouring CTA through distributed shared memory.  The result does not depend on the schedule
  * (the same arithmetic per node).  By default the library times every
  * schedule that fits on the first sweep run outside a stream capture (over
  * a sample of pairs, on a scratch intensity it allocates and frees there)

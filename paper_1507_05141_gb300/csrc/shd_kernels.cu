@@ -736,391 +736,6 @@ __global__ void __launch_bounds__(1024, 1) k_sweep_pipe(Prob<T> P, T *__restrict
 }
 
 // -------------------------------------------------------------------------
-// a4, FP32 with two previous-plane buffers: plane s reads the state of plane
-// s-1 from one float4 buffer (I, S, chi of a node) and writes its own into
-// the other, so one barrier per plane suffices: it makes plane s-1's state
-// and the copies of plane s visible, and every read of the buffer plane s
-// overwrites (plane s-2's) is done by then.  The inputs of plane s+1 stream
-// into a two-stage ring as in k_sweep_pipe (16-byte copies; a plane that
-// does not start on a 16-byte boundary is copied as its aligned cover and
-// read from its offset in the slot, so grids of any size keep the 16-byte
-// copies); with CB (aligned planes only) the moving-piece bits are read
-// from global memory when a plane's copies are issued.
-// -------------------------------------------------------------------------
-// One (ordinate, group) pair of the plane sweep by the CTA (tune_stride > 0,
-// schedule timing only: into column blockIdx.x of a scratch intensity).
-// reals by which p lies past the 16-byte boundary below it (p 4-byte aligned)
-__device__ __forceinline__ int shift16(const float *p)
-{
-    return (int)((reinterpret_cast<unsigned long long>(p) >> 2) & 3ull);
-}
-
-template <int U, bool CB, bool WIDE, int NT = 1024>
-__device__ __forceinline__ void sweep_pair_pp(const Prob<float> &P, float *__restrict__ I,
-                                              const float *__restrict__ eta, const float *__restrict__ chi,
-                                              const float *__restrict__ chi0L,
-                                              const unsigned long long *__restrict__ mbits, int npc, int nwin,
-                                              int pair, int tune_stride, unsigned char *smem_raw)
-{
-    const int k = pair / P.G;
-    const int g = pair - k * P.G;
-    const Ordinate o = P.ord[k];
-    const int dims[3] = {P.nx, P.ny, P.nz};
-    const int nd = dims[o.d], n1 = dims[o.e1], n2 = dims[o.e2];
-    const int plane = n1 * n2;
-    // planes whose start is not 16-byte aligned (grids with a plane or Nc
-    // not a multiple of 4) are copied as their aligned cover, up to 3 reals
-    // on either side: 4 reals of room past the rounded plane
-    const int pstride = ((plane + 3) & ~3) + 4;
-    float4 *Q = reinterpret_cast<float4 *>(smem_raw);              // [2][pstride]
-    float *ring = reinterpret_cast<float *>(Q + 2 * (size_t)pstride);  // [2][3][pstride]
-    const long long base = ((long long)k * P.G + g) * P.Nc;
-    if (tune_stride > 0) I += (long long)blockIdx.x * P.Nc - base;
-    const float *c0base = CB ? chi0L + ((long long)o.d * P.G + g) * P.Nc : nullptr;
-    const unsigned long long *mb = CB ? mbits + (size_t)o.d * nwin * npc : nullptr;
-    const float fr1 = (float)o.fr1, fr2 = (float)o.fr2, s = (float)o.s, kap = P.kappa;
-    const float w00 = (1.f - fr1) * (1.f - fr2), w10 = fr1 * (1.f - fr2), w01 = (1.f - fr1) * fr2, w11 = fr1 * fr2;
-    const float bc_iso = P.bc_mode == SHD_BC_ISO ? P.bc[g] : 0.f;
-    const bool bc_full = P.bc_mode == SHD_BC_FULL;
-    const int tid = threadIdx.x;
-
-    unsigned face = 0;
-    {
-        const int first1 = o.s1 > 0 ? 0 : n1 - 1, first2 = o.s2 > 0 ? 0 : n2 - 1;
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            int j = tid + NT * u;
-            int i1 = j / n2, i2 = j - i1 * n2;
-            if ((o.s1 != 0 && i1 == first1) || (o.s2 != 0 && i2 == first2)) face |= 1u << u;
-        }
-    }
-    const int d1 = o.s1 * n2, d2 = o.s2;
-    // the moving-node bits of this thread's chi pieces (plane <= U NT nodes,
-    // 4 a piece: at most MP pieces a thread) for the current 64-plane
-    // window, held in registers and reloaded when the window changes
-    constexpr int MP = (U + 3) / 4;
-    unsigned long long mw[MP];
-    int mwin = -1;
-
-    auto issue = [&](int step) {
-        if (step < nd) {
-            const int id = o.sd > 0 ? step : nd - 1 - step;
-            const long long pb = base + (long long)id * plane;
-            float *r = ring + (size_t)(step & 1) * 3 * pstride;
-            if constexpr (!CB) {
-                // the aligned cover of the plane in each array, shifted by
-                // the start's offset a within its 16 bytes (reals [a, a+plane)
-                // of the slot hold the plane)
-                const int aI = shift16(I + pb), aE = shift16(eta + pb), aC = shift16(chi + pb);
-                const float *gI = I + pb - aI, *gE = eta + pb - aE, *gC = chi + pb - aC;
-                const int nI = (aI + plane + 3) >> 2, nE = (aE + plane + 3) >> 2, nC = (aC + plane + 3) >> 2;
-                for (int q = tid; q < nI; q += NT) cp_async_n<16>(&r[q * 4], gI + q * 4);
-                for (int q = tid; q < nE; q += NT) cp_async_n<16>(&r[pstride + q * 4], gE + q * 4);
-                for (int q = tid; q < nC; q += NT) cp_async_n<16>(&r[2 * pstride + q * 4], gC + q * 4);
-                asm volatile("cp.async.commit_group;\n" ::);
-                return;
-            }
-            const int nv = plane / 4;  // 16-byte pieces per array (aligned planes)
-            for (int q = tid; q < nv; q += NT) cp_async_n<16>(&r[q * 4], &I[pb + q * 4]);
-            for (int q = tid; q < nv; q += NT) cp_async_n<16>(&r[pstride + q * 4], &eta[pb + q * 4]);
-            if (CB && (id >> 6) != mwin) {
-                mwin = id >> 6;
-#pragma unroll
-                for (int pi = 0; pi < MP; ++pi) {
-                    const int q = tid + pi * NT;
-                    mw[pi] = q < nv ? mb[(size_t)mwin * npc + q] : 0ull;
-                }
-            }
-#pragma unroll
-            for (int pi = 0; pi < MP; ++pi) {
-                const int q = tid + pi * NT;
-                if (q >= nv) break;
-                const int off = q * 4;
-                const float *src = chi + pb + off;
-                if (CB && !((mw[pi] >> (id & 63)) & 1ull)) src = c0base + (long long)id * plane + off;
-                cp_async_n<16>(&r[2 * pstride + off], src);
-            }
-        }
-        asm volatile("cp.async.commit_group;\n" ::);
-    };
-
-    issue(0);
-    for (int step = 0; step < nd; ++step) {
-        asm volatile("cp.async.wait_group 0;\n" ::);
-        __syncthreads();  // this plane's copies and the previous plane's state are visible
-        issue(step + 1);
-        const bool first = step == 0;
-        const int id = o.sd > 0 ? step : nd - 1 - step;
-        const long long pb = base + (long long)id * plane;
-        // per-plane bases of this thread's accesses: node u of the thread is
-        // at a constant offset NT u from each (the upwind ones are formed for
-        // every node but read only off the inflow faces)
-        const float *rI = ring + (size_t)(step & 1) * 3 * pstride + tid;
-        const float *rE = rI + pstride, *rC = rI + 2 * pstride;
-        if constexpr (!CB) {
-            rI += shift16(I + pb);
-            rE += shift16(eta + pb);
-            rC += shift16(chi + pb);
-        }
-        const float4 *qa = Q + (size_t)((step + 1) & 1) * pstride + tid;  // plane step - 1
-        const float4 *qb = qa - d1, *qc = qa - d2, *qd = qa - d1 - d2;
-        float4 *qn = Q + (size_t)(step & 1) * pstride + tid;               // plane step
-        float *ig = I + pb + tid;
-        const unsigned bnd = first ? ~0u : face;
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (tid + NT * u >= plane) break;
-            const float In = rI[NT * u];
-            const float ct = rC[NT * u] + kap;
-            const float st = ct > 0.f ? (rE[NT * u] + kap * In) * hw_rcp(ct) : 0.f;
-            float inew;
-            if ((bnd >> u) & 1u) {
-                inew = bc_full ? P.bc[pb + tid + NT * u] : bc_iso;
-            } else {
-                const float4 q00 = qa[NT * u], q10 = qb[NT * u], q01 = qc[NT * u], q11 = qd[NT * u];
-                const float iu = w00 * q00.x + w10 * q10.x + w01 * q01.x + w11 * q11.x;
-                const float su = w00 * q00.y + w10 * q10.y + w01 * q01.y + w11 * q11.y;
-                const float cu = w00 * q00.z + w10 * q10.z + w01 * q01.z + w11 * q11.z;
-                const float dtau = s * 0.5f * (cu + ct);
-                float ew, wp, wu;
-                if constexpr (WIDE) sc_weights<float>(dtau, ew, wp, wu);
-                else sc_weights_narrow_x2(dtau, ew, wp, wu);
-                inew = iu * ew + st * wp + su * wu;
-            }
-            qn[NT * u] = make_float4(inew, st, ct, 0.f);
-            ig[NT * u] = inew;
-        }
-    }
-    asm volatile("cp.async.wait_group 0;\n" ::);
-}
-
-// NT threads a CTA (1024, or 512 / 256 for small planes, 1024 / NT CTAs
-// an SM at the same 64 registers a thread)
-template <int U, bool CB, bool WIDE, int NT>
-__global__ void __launch_bounds__(NT, 1024 / NT) k_sweep_pp(Prob<float> P, float *__restrict__ I,
-                                                      const float *__restrict__ eta, const float *__restrict__ chi,
-                                                      const float *__restrict__ chi0L,
-                                                      const unsigned long long *__restrict__ mbits, int npc, int nwin,
-                                                      int tune_stride)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    // tune_stride > 0 (schedule timing only): CTA b sweeps pair b * tune_stride
-    // with its intensity in column b of a scratch array I [b][Nc]
-    const int pair = tune_stride > 0 ? (int)blockIdx.x * tune_stride : (int)blockIdx.x;
-    sweep_pair_pp<U, CB, WIDE, NT>(P, I, eta, chi, chi0L, mbits, npc, nwin, pair, tune_stride, smem_raw);
-}
-
-// The plane sweeps of a batch of problems in one persistent launch: CTAs
-// walk the work list of every problem's (ordinate, group) pairs (problem p
-// owns items [item0, item0 + N G)), each item as k_sweep_pp sweeps it, with
-// the problem's own fields and arrays.  One launch per class of problems
-// that share the kernel's variant (U, CB, WIDE).
-template <int U, bool CB, bool WIDE>
-__global__ void __launch_bounds__(1024, 1) k_sweep_batch(const SweepBatchProb *__restrict__ bp, int nprob,
-                                                         long long nitems)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    for (long long it = blockIdx.x; it < nitems; it += gridDim.x) {
-        int lo = 0, hi = nprob - 1;  // the last problem whose first item is <= it
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (bp[mid].item0 <= it) lo = mid;
-            else hi = mid - 1;
-        }
-        const SweepBatchProb &b = bp[lo];
-        __syncthreads();  // the previous item's reads of the shared buffers are done
-        sweep_pair_pp<U, CB, WIDE>(b.P, b.I, b.eta, b.chi, b.chi0L, b.mbits, b.npc, b.nwin, (int)(it - b.item0), 0,
-                                   smem_raw);
-    }
-}
-
-// -------------------------------------------------------------------------
-// a4, FP32, one plane split over a cluster of C CTAs: CTA r of the cluster
-// owns rows [r R, r R + R) of the plane (R rows of the in-plane axis e1, a
-// contiguous block of the sweep layout) and keeps the two previous-plane
-// buffers of k_sweep_pp for them only.  Upwind neighbours one row back that
-// belong to the neighbouring CTA (the first row of a CTA when n sweeps
-// towards +e1, the last when towards -e1) are read from that CTA's buffer
-// through distributed shared memory.  One cluster barrier per plane orders
-// the buffers exactly as k_sweep_pp's block barrier does, now across the
-// cluster.  Smaller CTAs let two or more clusters share an SM, so one
-// cluster's barrier wait overlaps another's compute; planes larger than one
-// CTA's shared memory fit across the cluster.  Every CTA runs every barrier
-// (no early exit) and a final one keeps its buffers alive until the peers'
-// last reads are done.  At 384 threads (three nodes a thread) the register
-// cap is 56, so three CTAs share an SM: one more cluster's compute under
-// each barrier wait.
-// -------------------------------------------------------------------------
-template <int U, bool CB, bool WIDE, int NT>
-__global__ void __launch_bounds__(NT, NT == 384 ? 3 : 1024 / NT) k_sweep_cl(Prob<float> P, float *__restrict__ I, const float *__restrict__ eta,
-                                                 const float *__restrict__ chi, const float *__restrict__ chi0L,
-                                                 const unsigned long long *__restrict__ mbits, int npc, int nwin,
-                                                 int pstride, int tune_stride)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    cg::cluster_group cl = cg::this_cluster();
-    const int C = (int)cl.num_blocks();
-    const int r = (int)cl.block_rank();
-    // tune_stride > 0 (schedule timing only): cluster b sweeps pair b *
-    // tune_stride with its intensity in column b of a scratch array I [b][Nc]
-    const int cidx = (int)blockIdx.x / C;
-    const int pair = tune_stride > 0 ? cidx * tune_stride : cidx;
-    const int k = pair / P.G;
-    const int g = pair - k * P.G;
-    const Ordinate o = P.ord[k];
-    const int dims[3] = {P.nx, P.ny, P.nz};
-    const int nd = dims[o.d], n1 = dims[o.e1], n2 = dims[o.e2];
-    const int plane = n1 * n2;
-    // rows per CTA: ceil(n1 / C), rounded up so every CTA's block of the
-    // layout starts on a 16-byte boundary
-    int R = (n1 + C - 1) / C;
-    const int q4 = (n2 & 3) == 0 ? 1 : ((n2 & 1) == 0 ? 2 : 4);
-    R = (R + q4 - 1) / q4 * q4;
-    const int row0 = r * R;
-    const int nrows = row0 >= n1 ? 0 : (n1 - row0 < R ? n1 - row0 : R);
-    const int nloc = nrows * n2;
-    const int j0 = row0 * n2;
-    float4 *Q = reinterpret_cast<float4 *>(smem_raw);                  // [2][pstride]
-    float *ring = reinterpret_cast<float *>(Q + 2 * (size_t)pstride);  // [2][3][pstride]
-    const long long base = ((long long)k * P.G + g) * P.Nc;
-    if (tune_stride > 0) I += (long long)cidx * P.Nc - base;
-    const float *c0base = CB ? chi0L + ((long long)o.d * P.G + g) * P.Nc : nullptr;
-    const unsigned long long *mb = CB ? mbits + (size_t)o.d * nwin * npc : nullptr;
-    const float fr1 = (float)o.fr1, fr2 = (float)o.fr2, s = (float)o.s, kap = P.kappa;
-    const float w00 = (1.f - fr1) * (1.f - fr2), w10 = fr1 * (1.f - fr2), w01 = (1.f - fr1) * fr2, w11 = fr1 * fr2;
-    const float bc_iso = P.bc_mode == SHD_BC_ISO ? P.bc[g] : 0.f;
-    const bool bc_full = P.bc_mode == SHD_BC_FULL;
-    const int tid = threadIdx.x;
-    // the CTA holding the row one step upwind of this CTA's boundary row
-    const int pr = o.s1 > 0 ? r - 1 : (o.s1 < 0 ? r + 1 : -1);
-    const bool has_peer = pr >= 0 && pr < C;
-    float4 *Qpeer = has_peer ? cl.map_shared_rank(Q, pr) : Q;
-    const int jpeer = has_peer ? pr * R * n2 : 0;  // first node of the peer's block
-
-    // bit u of `face`: node j0 + tid + NT u is on an inflow face of an
-    // in-plane axis; bit u of `halo`: its row-upwind neighbours are the peer's
-    unsigned face = 0, halo = 0;
-    {
-        const int first1 = o.s1 > 0 ? 0 : n1 - 1, first2 = o.s2 > 0 ? 0 : n2 - 1;
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int jl = tid + NT * u;
-            if (jl >= nloc) break;
-            const int i1 = (j0 + jl) / n2, i2 = (j0 + jl) - i1 * n2;
-            if ((o.s1 != 0 && i1 == first1) || (o.s2 != 0 && i2 == first2)) face |= 1u << u;
-            const int jn = jl - o.s1 * n2;
-            if (jn < 0 || jn >= nloc) halo |= 1u << u;
-        }
-    }
-    const int d1 = o.s1 * n2, d2 = o.s2;
-    // moving-node bits of this thread's chi pieces, as in k_sweep_pp
-    constexpr int MP = (U + 3) / 4;
-    unsigned long long mw[MP];
-    int mwin = -1;
-
-    auto issue = [&](int step) {
-        if (step < nd) {
-            const int id = o.sd > 0 ? step : nd - 1 - step;
-            const long long pb = base + (long long)id * plane + j0;
-            float *rg = ring + (size_t)(step & 1) * 3 * pstride;
-            const int nv = nloc / 4;  // 16-byte pieces per array
-            for (int q = tid; q < nv; q += NT) cp_async_n<16>(&rg[q * 4], &I[pb + q * 4]);
-            for (int q = tid; q < nv; q += NT) cp_async_n<16>(&rg[pstride + q * 4], &eta[pb + q * 4]);
-            if (CB && (id >> 6) != mwin) {
-                mwin = id >> 6;
-#pragma unroll
-                for (int pi = 0; pi < MP; ++pi) {
-                    const int q = tid + pi * NT;
-                    mw[pi] = q < nv ? mb[(size_t)mwin * npc + (j0 >> 2) + q] : 0ull;
-                }
-            }
-#pragma unroll
-            for (int pi = 0; pi < MP; ++pi) {
-                const int q = tid + pi * NT;
-                if (q >= nv) break;
-                const int off = q * 4;
-                const float *src = chi + pb + off;
-                if (CB && !((mw[pi] >> (id & 63)) & 1ull)) src = c0base + (long long)id * plane + j0 + off;
-                cp_async_n<16>(&rg[2 * pstride + off], src);
-            }
-        }
-        asm volatile("cp.async.commit_group;\n" ::);
-    };
-
-    // The cluster barrier is split: a thread arrives (release: its writes of
-    // the plane buffer and its landed copies) and then stores the previous
-    // plane's intensities to global memory before it waits, so that a release
-    // never waits for that plane's global stores; the next arrival covers
-    // them a plane later.
-    float inew_u[U];
-    long long pb_prev = -1;
-    auto store_prev = [&]() {
-        if (pb_prev < 0) return;
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int j = tid + NT * u;
-            if (j >= nloc) break;
-            I[pb_prev + j] = inew_u[u];
-        }
-    };
-    issue(0);
-    for (int step = 0; step < nd; ++step) {
-        asm volatile("cp.async.wait_group 0;\n" ::);
-        // this plane's copies and the cluster's previous-plane state are visible after the wait
-        asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
-        store_prev();
-        asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-        issue(step + 1);
-        const float *rg = ring + (size_t)(step & 1) * 3 * pstride;
-        const size_t pprev = (size_t)((step + 1) & 1) * pstride;
-        const float4 *Qp = Q + pprev;                   // plane step - 1, this CTA's rows
-        const float4 *Qr = Qpeer + pprev;               // plane step - 1, the peer's rows
-        float4 *Qn = Q + (size_t)(step & 1) * pstride;  // plane step
-        const bool first = step == 0;
-        const int id = o.sd > 0 ? step : nd - 1 - step;
-        const long long pb = base + (long long)id * plane + j0;
-        pb_prev = pb;
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int j = tid + NT * u;
-            if (j >= nloc) break;
-            const float In = rg[j];
-            const float ct = rg[2 * pstride + j] + kap;
-            const float st = ct > 0.f ? (rg[pstride + j] + kap * In) * hw_rcp(ct) : 0.f;
-            float inew;
-            if (first || ((face >> u) & 1u)) {
-                inew = bc_full ? P.bc[pb + j] : bc_iso;
-            } else {
-                const float4 q00 = Qp[j], q01 = Qp[j - d2];
-                float4 q10, q11;
-                if ((halo >> u) & 1u) {
-                    const int jr = j0 + j - d1 - jpeer;  // the peer's local index
-                    q10 = Qr[jr];
-                    q11 = Qr[jr - d2];
-                } else {
-                    q10 = Qp[j - d1];
-                    q11 = Qp[j - d1 - d2];
-                }
-                const float iu = w00 * q00.x + w10 * q10.x + w01 * q01.x + w11 * q11.x;
-                const float su = w00 * q00.y + w10 * q10.y + w01 * q01.y + w11 * q11.y;
-                const float cu = w00 * q00.z + w10 * q10.z + w01 * q01.z + w11 * q11.z;
-                const float dtau = s * 0.5f * (cu + ct);
-                float ew, wp, wu;
-                if constexpr (WIDE) sc_weights<float>(dtau, ew, wp, wu);
-                else sc_weights_narrow_x2(dtau, ew, wp, wu);
-                inew = iu * ew + st * wp + su * wu;
-            }
-            Qn[j] = make_float4(inew, st, ct, 0.f);
-            inew_u[u] = inew;
-        }
-    }
-    asm volatile("cp.async.wait_group 0;\n" ::);
-    asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
-    store_prev();  // the last plane
-    asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");  // the peers' reads of this CTA's buffers are done
-}
-
-// -------------------------------------------------------------------------
 // a4 with the cubic Bezier short characteristic (Sec. 2), any precision, one
 // 1024-thread CTA per (ordinate, group).  Besides the upwind point U the
 // source's end derivatives need the downwind point D = P + s n on the next
@@ -2064,7 +1679,7 @@ static cudaError_t launch_sweep_npt(const shd_ctx *ctx, T *I, const T *eta, cons
 // Optical depth of one short-characteristic step is at most s_max chi~_max
 // with chi~ = chi_lab + kappa and chi_lab <= chi0_max D_max, D = Gamma - u.n <
 // 2 Gamma (R17): true when that stays within kTauPlain.
-static bool sweep_tau_bounded(const shd_ctx *c)
+bool sweep_tau_bounded(const shd_ctx *c)
 {
     double smax = 0;
     for (const Ordinate &o : c->h_ord) smax = o.s > smax ? o.s : smax;
@@ -2091,250 +1706,6 @@ static cudaError_t launch_sweep_pipe(const shd_ctx *ctx, T *I, const T *eta, con
     return cudaGetLastError();
 }
 
-// shared memory of the FP32 two-buffer sweep: two float4 planes and the
-// 2-stage ring of the three inputs
-static size_t sweep_pp_smem_bytes(const shd_ctx *c)
-{
-    size_t ps = (((size_t)sweep_plane_max(c) + 3) & ~(size_t)3) + 4;  // k_sweep_pp's plane stride
-    return sizeof(float) * ps * 14;
-}
-
-template <int U, int NT>
-static cudaError_t launch_sweep_pp(const shd_ctx *ctx, float *I, const float *eta, const float *chi, cudaStream_t st,
-                                   bool bits, bool wide, unsigned nblocks, int tune_stride)
-{
-    Prob<float> P = make_prob<float>(ctx);
-    const float *c0L = bits ? (const float *)ctx->d_chi0L : nullptr;
-    const unsigned long long *mb = bits ? ctx->d_mbits : nullptr;
-    const size_t sm = sweep_pp_smem_bytes(ctx);
-    auto kern = bits ? (wide ? k_sweep_pp<U, true, true, NT> : k_sweep_pp<U, true, false, NT>)
-                     : (wide ? k_sweep_pp<U, false, true, NT> : k_sweep_pp<U, false, false, NT>);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    kern<<<nblocks, NT, sm, st>>>(P, I, eta, chi, c0L, mb, ctx->mbits_npc, ctx->mbits_nwin, tune_stride);
-    note_launch();
-    return cudaGetLastError();
-}
-
-// ---- schedules of the FP32 plane sweep ------------------------------------
-// A schedule splits every plane over a cluster of C CTAs of NT threads, U
-// nodes a thread (C = 1: k_sweep_pp, one CTA of NT = 1024, 512 or 256
-// threads a plane).
-
-struct SweepSched {
-    int C = 0, NT = 0, U = 0, pstride = 0;
-    size_t smem = 0;
-};
-
-// rows of a plane per CTA of a C-CTA cluster (the kernel's own rule)
-static int sweep_rows_per_cta(int n1, int n2, int C)
-{
-    int R = (n1 + C - 1) / C;
-    const int q4 = (n2 & 3) == 0 ? 1 : ((n2 & 1) == 0 ? 2 : 4);
-    return (R + q4 - 1) / q4 * q4;
-}
-
-// Nodes per CTA of the largest class plane under a C-CTA split.
-static int sweep_nloc_max(const shd_ctx *c, int C)
-{
-    const int dims[3] = {c->nx, c->ny, c->nz};
-    bool seen[3] = {false, false, false};
-    int m = 0;
-    for (const Ordinate &o : c->h_ord) {
-        if (seen[o.d]) continue;
-        seen[o.d] = true;
-        const int n1 = dims[o.e1], n2 = dims[o.e2];
-        const int R = sweep_rows_per_cta(n1, n2, C);
-        const int nl = (R < n1 ? R : n1) * n2;
-        m = nl > m ? nl : m;
-    }
-    return m;
-}
-
-template <int U, int NT>
-static cudaError_t launch_sweep_cl_t(const shd_ctx *ctx, const SweepSched &sc, float *I, const float *eta,
-                                     const float *chi, cudaStream_t st, bool bits, bool wide, int nclusters,
-                                     int tune_stride)
-{
-    Prob<float> P = make_prob<float>(ctx);
-    const float *c0L = bits ? (const float *)ctx->d_chi0L : nullptr;
-    const unsigned long long *mb = bits ? ctx->d_mbits : nullptr;
-    auto kern = bits ? (wide ? k_sweep_cl<U, true, true, NT> : k_sweep_cl<U, true, false, NT>)
-                     : (wide ? k_sweep_cl<U, false, true, NT> : k_sweep_cl<U, false, false, NT>);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sc.smem);
-    if (e != cudaSuccess) return e;
-    // the whole unified L1 as shared memory, so that the CTAs the register
-    // budget allows (three of 384 threads at 56 registers) also fit there
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    if (e != cudaSuccess) return e;
-    if (sc.C > 8) {  // 16-CTA clusters are beyond the portable size: opted in per kernel
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e != cudaSuccess) return e;
-    }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(nclusters * sc.C));
-    cfg.blockDim = dim3(NT);
-    cfg.dynamicSmemBytes = sc.smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)sc.C;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, kern, P, I, eta, chi, c0L, mb, ctx->mbits_npc, ctx->mbits_nwin, sc.pstride,
-                           tune_stride);
-    note_launch();
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
-}
-
-// Run schedule sc over `n` (ordinate, group) pairs (all of them, or every
-// tune_stride-th into a scratch intensity when timing).
-static cudaError_t run_sweep_sched(const shd_ctx *ctx, const SweepSched &sc, float *I, const float *eta,
-                                   const float *chi, cudaStream_t st, bool bits, bool wide, int n, int tune_stride)
-{
-    if (sc.C == 1) {
-#define SHD_PP(Uv, NTv) \
-    if (sc.U == Uv && sc.NT == NTv) return launch_sweep_pp<Uv, NTv>(ctx, I, eta, chi, st, bits, wide, (unsigned)n, tune_stride);
-        SHD_PP(1, 1024) SHD_PP(2, 1024) SHD_PP(4, 1024)
-        SHD_PP(1, 512) SHD_PP(2, 512) SHD_PP(4, 512)
-        SHD_PP(1, 256) SHD_PP(2, 256) SHD_PP(4, 256)
-#undef SHD_PP
-        return cudaErrorInvalidConfiguration;
-    }
-#define SHD_CL(NTv, Uv) \
-    if (sc.NT == NTv && sc.U == Uv) return launch_sweep_cl_t<Uv, NTv>(ctx, sc, I, eta, chi, st, bits, wide, n, tune_stride);
-    SHD_CL(256, 2) SHD_CL(256, 4) SHD_CL(384, 3) SHD_CL(512, 2) SHD_CL(512, 4) SHD_CL(768, 3) SHD_CL(1024, 2)
-    SHD_CL(1024, 4)
-#undef SHD_CL
-    return cudaErrorInvalidConfiguration;
-}
-
-// The schedule (C, NT) with its U, buffer stride and shared memory, if it
-// fits this problem; false otherwise.
-template <class T>
-static bool sweep_vec(const shd_ctx *ctx);
-
-static bool sweep_sched_make(const shd_ctx *c, int C, int NT, SweepSched &sc)
-{
-    sc = SweepSched();
-    const size_t limit = 227 * 1024;
-    if (C == 1) {  // any grid: k_sweep_pp copies unaligned planes as their aligned cover
-        if (NT != 1024 && NT != 512 && NT != 256) return false;
-        const int pm = sweep_plane_max(c);
-        const int u = (pm + NT - 1) / NT;
-        if (u > 4 || sweep_pp_smem_bytes(c) > limit) return false;
-        // smaller CTAs only where they keep more than half their threads busy
-        if (NT < 1024 && pm <= NT / 2) return false;
-        if (NT < 1024 && (1024 / NT) * sweep_pp_smem_bytes(c) > limit) return false;  // their CTAs share the SM
-        sc.C = 1; sc.NT = NT; sc.U = u <= 1 ? 1 : (u <= 2 ? 2 : 4);
-        sc.smem = sweep_pp_smem_bytes(c);
-        return true;
-    }
-    if (C != 2 && C != 4 && C != 8 && C != 16) return false;
-    if (!sweep_vec<float>(c)) return false;  // the cluster sweep's blocks need 16-byte aligned planes
-    if (NT != 256 && NT != 384 && NT != 512 && NT != 768 && NT != 1024) return false;
-    const int nl = sweep_nloc_max(c, C);
-    int U = 0;
-    if (NT == 384 || NT == 768) {
-        // three nodes a thread: blocks that 2 or 4 a thread would fit loosely
-        // (1152 nodes: 384 x 3 exactly, against 512 x 4 with a third idle)
-        if (nl <= 2 * NT || nl > 3 * NT) return false;
-        U = 3;
-    } else if (nl <= 2 * NT) U = 2;
-    else if (nl <= 4 * NT) U = 4;
-    else return false;
-    if (nl <= NT / 2) return false;  // half the threads or more would idle
-    sc.C = C; sc.NT = NT; sc.U = U;
-    sc.pstride = (nl + 3) & ~3;
-    sc.smem = sizeof(float) * (size_t)sc.pstride * 14;
-    return sc.smem <= limit;
-}
-
-// Every schedule that fits, k_sweep_pp's first.
-static std::vector<SweepSched> sweep_candidates(const shd_ctx *c)
-{
-    std::vector<SweepSched> v;
-    SweepSched sc;
-    if (sweep_sched_make(c, 1, 1024, sc)) v.push_back(sc);
-    for (int NT : {512, 256})
-        if (sweep_sched_make(c, 1, NT, sc)) v.push_back(sc);
-    for (int C : {2, 4, 8, 16})
-        for (int NT : {256, 384, 512, 768, 1024})
-            if (sweep_sched_make(c, C, NT, sc)) v.push_back(sc);
-    return v;
-}
-
-// The FP32 sweep's schedule: forced, chosen earlier, or chosen now by timing
-// each candidate (one warm-up and three timed launches over every
-// tune_stride-th pair, intensity in a scratch array) when the stream is not
-// being captured; under capture without a choice, the first candidate.
-static bool sweep_schedule(const shd_ctx *cc, cudaStream_t st, const float *eta, const float *chi, bool bits,
-                           bool wide, SweepSched &out)
-{
-    shd_ctx *c = const_cast<shd_ctx *>(cc);  // the choice is a cache of the context
-    if (c->sweep_force_C > 0) return sweep_sched_make(c, c->sweep_force_C, c->sweep_force_NT, out);
-    if (c->sweep_C > 0 && sweep_sched_make(c, c->sweep_C, c->sweep_NT, out)) return true;
-    std::vector<SweepSched> cand = sweep_candidates(c);
-    if (cand.empty()) return false;
-    out = cand[0];
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return true;
-    c->sweep_ntune = 0;
-    if (cand.size() > 1) {
-        int sms = 0;
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess || sms <= 0)
-            sms = 148;
-        const int npairs = c->N * c->G;
-        const int n = npairs < 4 * sms ? npairs : 4 * sms;
-        const int stride = npairs / n;
-        float *scratch = nullptr;
-        // (+16 bytes: the aligned cover of an unaligned last plane)
-        if (cudaMalloc(&scratch, sizeof(float) * (size_t)n * c->Nc + 16) != cudaSuccess) {
-            cudaGetLastError();
-            return true;  // no room to time them: the first candidate
-        }
-        cudaMemsetAsync(scratch, 0, sizeof(float) * (size_t)n * c->Nc, st);
-        cudaEvent_t e0, e1;
-        cudaEventCreate(&e0);
-        cudaEventCreate(&e1);
-        float best = 1e30f;
-        for (const SweepSched &sc : cand) {
-            float ms = 1e30f;
-            if (run_sweep_sched(c, sc, scratch, eta, chi, st, bits, wide, n, stride) == cudaSuccess) {
-                cudaEventRecord(e0, st);
-                bool ok = true;
-                for (int r = 0; r < 3 && ok; ++r)
-                    ok = run_sweep_sched(c, sc, scratch, eta, chi, st, bits, wide, n, stride) == cudaSuccess;
-                cudaEventRecord(e1, st);
-                if (ok && cudaEventSynchronize(e1) == cudaSuccess) {
-                    cudaEventElapsedTime(&ms, e0, e1);
-                    ms /= 3.f;
-                }
-            }
-            cudaGetLastError();  // a candidate that cannot launch here is skipped
-            if (c->sweep_ntune < 16) {
-                c->sweep_tune[c->sweep_ntune][0] = (float)sc.C;
-                c->sweep_tune[c->sweep_ntune][1] = (float)sc.NT;
-                c->sweep_tune[c->sweep_ntune][2] = ms;
-                c->sweep_ntune++;
-            }
-            if (ms < best) {
-                best = ms;
-                out = sc;
-            }
-        }
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
-        cudaFree(scratch);
-    }
-    c->sweep_C = out.C;
-    c->sweep_NT = out.NT;
-    return true;
-}
-
 // shared memory of the pipelined sweep: previous plane (4 reals a node in
 // FP32, 3 in FP64) + 2-stage ring of the three inputs, each array padded to
 // a multiple of 4 reals
@@ -2353,85 +1724,20 @@ static bool sweep_vec(const shd_ctx *ctx)
            ((long long)ctx->nx * ctx->nz) % V == 0;
 }
 
-size_t sweep_batch_smem(const shd_ctx *c) { return sweep_pp_smem_bytes(c); }
+bool sweep_planes_aligned(const shd_ctx *ctx) { return sweep_vec<float>(ctx); }
 
-// the descriptor of problem c as its own sweep launch would see it
-void sweep_batch_fill(const shd_ctx *c, SweepBatchProb &d, long long item0)
-{
-    d.P = make_prob<float>(c);
-    d.I = (float *)c->d_I;
-    d.eta = (const float *)c->d_eta;
-    d.chi = (const float *)c->d_chi;
-    const bool bits = sweep_uses_chi0L<float>(c);
-    d.chi0L = bits ? (const float *)c->d_chi0L : nullptr;
-    d.mbits = bits ? c->d_mbits : nullptr;
-    d.npc = c->mbits_npc;
-    d.nwin = c->mbits_nwin;
-    d.cb = bits ? 1 : 0;
-    d.wide = sweep_tau_bounded(c) ? 0 : 1;
-    d.item0 = item0;
-}
-
-int sweep_batch_class(const shd_ctx *c)
-{
-    if (c->precision == SHD_FP64 || c->integrator != SHD_SC_LINEAR) return 0;
-    SweepSched sc;
-    if (!sweep_sched_make(c, 1, 1024, sc)) return 0;
-    if (c->sweep_force_C > 0 && !(c->sweep_force_C == 1 && c->sweep_force_NT == 1024)) return 0;
-    if (c->sweep_force_C <= 0 && c->sweep_C > 0 && !(c->sweep_C == 1 && c->sweep_NT == 1024)) {
-        // another schedule won the problem's timing: it joins only if the
-        // 1024-thread one-CTA sweep (the batch's) timed within 3 % of that
-        float pp = -1.f, best = 1e30f;
-        for (int k = 0; k < c->sweep_ntune; ++k) {
-            if (c->sweep_tune[k][0] == 1.f && c->sweep_tune[k][1] == 1024.f) pp = c->sweep_tune[k][2];
-            best = fminf(best, c->sweep_tune[k][2]);
-        }
-        if (!(pp > 0.f && pp <= 1.03f * best)) return 0;
-    }
-    // class: U (bits 0-2), chi0 table (bit 3), compensated exponential (bit 4)
-    return sc.U | (sweep_uses_chi0L<float>(c) ? 8 : 0) | (sweep_tau_bounded(c) ? 0 : 16);
-}
-
-cudaError_t launch_sweep_batch(int cls, const SweepBatchProb *d_probs, int nprob, long long nitems, size_t smem,
-                               int device, cudaStream_t st)
-{
-    if (nprob <= 0 || nitems <= 0) return cudaSuccess;
-    using KB = void (*)(const SweepBatchProb *, int, long long);
-    const int U = cls & 7;
-    const bool cb = (cls & 8) != 0, wide = (cls & 16) != 0;
-    KB kern;
-    if (U <= 1) kern = cb ? (wide ? k_sweep_batch<1, true, true> : k_sweep_batch<1, true, false>)
-                          : (wide ? k_sweep_batch<1, false, true> : k_sweep_batch<1, false, false>);
-    else if (U <= 2) kern = cb ? (wide ? k_sweep_batch<2, true, true> : k_sweep_batch<2, true, false>)
-                               : (wide ? k_sweep_batch<2, false, true> : k_sweep_batch<2, false, false>);
-    else kern = cb ? (wide ? k_sweep_batch<4, true, true> : k_sweep_batch<4, true, false>)
-                   : (wide ? k_sweep_batch<4, false, true> : k_sweep_batch<4, false, false>);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int nsm = 0, per = 0;
-    if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || nsm <= 0) nsm = 148;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, 1024, smem) != cudaSuccess || per < 1) per = 1;
-    long long grid = (long long)nsm * per;  // persistent: every CTA that fits at once
-    if (grid > nitems) grid = nitems;
-    kern<<<(unsigned)grid, 1024, smem, st>>>(d_probs, nprob, nitems);
-    note_launch();
-    return cudaGetLastError();
-}
-
-// (C, NT) is a schedule of the FP32 plane sweep for this problem
-bool sweep_schedule_valid(const shd_ctx *c, int C, int NT)
-{
-    SweepSched sc;
-    return c->precision != SHD_FP64 && sweep_sched_make(c, C, NT, sc);
-}
-
+// chi at rest from the chi0 table: where a kernel that reads it sweeps the
+// problem (128^2 planes, which only the cluster schedules sweep, then read
+// 12 + 4 f B a node instead of 16, f the share of pieces that move)
 template <class T>
 bool sweep_uses_chi0L(const shd_ctx *ctx)
 {
     if (ctx->integrator != SHD_SC_LINEAR) return false;  // the Bezier sweep reads every chi_lab
+    if (!ctx->d_chi0L || !ctx->d_mbits || !sweep_vec<T>(ctx)) return false;
     const int u = (sweep_plane_max(ctx) + 1023) / 1024;
-    return ctx->d_chi0L && ctx->d_mbits && sweep_vec<T>(ctx) && u <= 8 &&
-           sweep_pipe_smem_bytes(ctx) + sizeof(unsigned long long) * (size_t)ctx->mbits_npc <= 227 * 1024;
+    if (u <= 8 && sweep_pipe_smem_bytes(ctx) + sizeof(unsigned long long) * (size_t)ctx->mbits_npc <= 227 * 1024)
+        return true;
+    return sizeof(T) == 4 && sweep_has_schedule(ctx);
 }
 
 // use_chi0L: the per-ordinate chi is only valid on the pieces that hold a
@@ -2477,14 +1783,9 @@ cudaError_t launch_sweep(const shd_ctx *ctx, T *I, const T *eta, const T *chi, c
     }
     size_t smp = sweep_pipe_smem_bytes(ctx);
     if constexpr (sizeof(T) == 4) {
-        {
-            const bool bits = use_chi0L && sweep_uses_chi0L<T>(ctx);
-            const bool wide = !sweep_tau_bounded(ctx);
-            SweepSched sc;
-            if (sweep_schedule(ctx, st, (const float *)eta, (const float *)chi, bits, wide, sc))
-                return run_sweep_sched(ctx, sc, (float *)I, (const float *)eta, (const float *)chi, st, bits, wide,
-                                       ctx->N * ctx->G, 0);
-        }
+        bool ran = false;
+        const cudaError_t e = launch_sweep_f(ctx, I, eta, chi, st, use_chi0L && sweep_uses_chi0L<T>(ctx), &ran);
+        if (ran || e != cudaSuccess) return e;
     }
     if (smp <= 227 * 1024) {
         const bool vec = sweep_vec<T>(ctx);
