@@ -879,7 +879,7 @@ int ensure_remap_tables(shd_ctx *c, cudaStream_t st)
     return SHD_OK;
 }
 
-// The segment transform (MIXED) stores chi_lab only where a node moves.  The
+// The segment transform (MIXED) and FP32's a3 store chi_lab only where a node moves.  The
 // sweep reads chi at rest from the chi0 layout table where it can (aligned
 // rows, c0L); elsewhere -- other sweep kernels, or rows not a multiple of 4
 // nodes, where a 4-node piece may straddle a moving and a resting row -- it
@@ -888,13 +888,13 @@ template <class T>
 bool rest_chi_kept(const shd_ctx *c)
 {
     if constexpr (sizeof(T) == 4)
-        return c->precision == SHD_MIXED && seg_usable(c) && c->d_chi0L && c->d_chi_dirty;
+        return ((c->precision == SHD_MIXED && seg_usable(c)) || sh2lab_f32_usable(c)) && c->d_chi0L && c->d_chi_dirty;
     return false;
 }
 template <class T>
 bool rest_chi_read(const shd_ctx *c)
 {
-    return rest_chi_kept<T>(c) && (!sweep_uses_chi0L<T>(c) || seg_manual(c));
+    return rest_chi_kept<T>(c) && (!sweep_uses_chi0L<T>(c) || c->nx % 4 != 0 || c->ny % 4 != 0);
 }
 
 // The fill of chi_lab at rest on st where the sweep reads it and chi0 or the

@@ -21,6 +21,7 @@
 // spaced in log energy they replace the bracket search by a constant shift.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "shd_internal.cuh"
@@ -206,218 +207,475 @@ __global__ void __launch_bounds__(256) k_sh2lab_tile(Prob<T> P, const T *__restr
 }
 
 // -------------------------------------------------------------------------
-// Persistent forms (used when the right-hand matrix fits in shared memory):
-// one CTA per SM loads W Y (project) or Y (sh2lab) once and then walks the
-// (tile, group) work items, so the matrix crosses L2 once per SM instead of
-// once per item.  A chunks are double-buffered with cp.async.
+// Single precision.  Both contractions are bound by the FP32 FMA rate (about
+// 65 TFLOP/s reachable; 2 x 65.5 kflop per node and group at L = 7), so the
+// tiles are chosen for FMAs per shared-memory load: 16 x TN (a1) and 4 x 16
+// (a3) register tiles, 80 and 64 FMAs per 9 and 5 loads at L = 7, operands
+// streamed by 16-byte cp.async (a1) or resident (a3).  48^3, 16 groups, 512
+// ordinates: a1 4.5 and a3 6.5 ms a call (23.2 and 11.9 ms for the 4 x 5 and
+// 8 x 4 tiles, with 4-byte copies and index arithmetic an element, that
+// these replaced).
 // -------------------------------------------------------------------------
-__device__ inline void cp_async4(void *smem, const void *gmem)
+__device__ inline void cp_async4(void *smem, const void *gmem, bool on)
 {
-    unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem));
+    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(s), "l"(gmem), "r"(on ? 4 : 0));
+}
+__device__ inline void cp_async16(void *smem, const void *gmem, bool on)
+{
+    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(s), "l"(gmem), "r"(on ? 16 : 0));
 }
 __device__ inline void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
 template <int N>
 __device__ inline void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
 
-// a1, persistent: 256 threads = 16 row groups of 4 rows x 16 column groups of
-// TC contiguous columns (NB = 16 TC).  Shared: Bs[N][NB] + As[2][KC][64].
-template <int TC>
-__global__ void __launch_bounds__(256, 1) k_project_persist(Prob<float> P, const float *__restrict__ I,
-                                                            const float *__restrict__ I0, float *__restrict__ Ip,
-                                                            float *__restrict__ mom)
+// a1: [128 rows x N] x [N x 16 TN] per CTA of 128 threads = 8 row groups of 16
+// rows x 16 column groups (columns tc + 16 j).  ROWS = 0: the rows are two
+// bricks of the tile list (consecutive tiles) in one energy group, their
+// laboratory intensity in run order (VEC: rows of the grid are 16-byte
+// multiples, one copy per half run); moments of every node and I_lm of nodes
+// at rest are stored, and the laboratory intensity of moving nodes goes
+// node-major into nmo for their remap (from the tile in shared memory: a
+// separate transpose pass over the bricks took 1.2 ms a call).  The x-class
+// ordinates' runs go along y: their rows are read transposed.  ROWS = 1: 128
+// (moving node, group) rows of the node-major comoving intensity, I_lm of
+// moving nodes.
+constexpr int kPKC = 16, kPStages = 3, kPRow = 132;
+
+template <int TN, int ROWS, bool VEC>
+__global__ void __launch_bounds__(128, TN <= 5 ? 3 : 2) k_project_f32(Prob<float> P, const float *__restrict__ I,
+                                                                      float *__restrict__ Ip,
+                                                                      float *__restrict__ mom,
+                                                                      float *__restrict__ nmo, int nA, long long ntp)
 {
-    constexpr int R = 64, KC = 32, NB = 16 * TC, TR = 4;
+    constexpr int KC = kPKC, NBC = 16 * TN;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float *Bs = reinterpret_cast<float *>(smem_raw);        // [N][NB]
-    float *As = Bs + (size_t)P.N * NB;                       // [2][KC][R]
+    float *As = reinterpret_cast<float *>(smem_raw);  // [kPStages][KC][kPRow]
+    float *Bs = As + kPStages * KC * kPRow;            // [kPStages][KC][NBC]
     const int tid = threadIdx.x, tr = tid >> 4, tc = tid & 15;
-    const int NLM = P.NLM, N = P.N, G = P.G;
-    for (int e = tid; e < N * NB; e += 256) Bs[e] = P.Bproj[e];
-    const long long items = P.ntiles * G;
+    const int G = P.G, N = P.N, NLM = P.NLM, nx = P.nx, ny = P.ny, nz = P.nz;
     const int nchunk = (N + KC - 1) / KC;
-    for (long long w = blockIdx.x; w < items; w += gridDim.x) {
-        const long long tile = w / G;
-        const int g = (int)(w - tile * G);
-        const TileInfo ti = P.tiles[tile];
-        const int passes = (ti.flags & 1) ? 2 : 1;
-        for (int pass = 0; pass < passes; ++pass) {
-            // columns this pass needs: everything in pass 0, the SH part in pass 1
-            const int ncol = pass == 0 ? NB : NLM;
-            float acc[TR][TC];
+    // laboratory rows: tile pair fastest, so that CTAs in flight read
+    // neighbouring runs
+    const int g0 = ROWS ? 0 : (int)(blockIdx.x / ntp);
+    const long long t0 = ROWS ? 0 : 2 * (blockIdx.x - g0 * ntp);
+    const long long row0 = ROWS ? (long long)blockIdx.x * 128 : 0, nrows = P.nmoving * G;
+    // this thread's piece of every ordinate's tile (VEC: a half run; else a
+    // node): offsets in the z-, y- and x-class layouts
+    long long oz = 0, oy = 0, ox = 0;
+    bool inz = false, inx = false;
+    if constexpr (!ROWS) {
+        const int b = VEC ? (tid & 31) >> 4 : tid >> 6, j = VEC ? (tid >> 1) & 7 : (tid >> 3) & 7;
+        const int i = VEC ? 4 * (tid & 1) : tid & 7;
+        if (t0 + b < P.ntiles) {
+            const TileInfo ti = P.tiles[t0 + b];
+            const int x = ti.x0 + i, y = ti.y0 + j, xt = ti.x0 + j, yt = ti.y0 + i;
+            inz = x < nx && y < ny;
+            inx = xt < nx && yt < ny;
+            oz = ((long long)ti.z * ny + y) * nx + x;
+            oy = ((long long)y * nz + ti.z) * nx + x;
+            ox = ((long long)xt * nz + ti.z) * ny + yt;
+        }
+    }
+    // the node-major row of tile row `tid` when its node moves
+    float *nrow = nullptr;
+    if constexpr (!ROWS) {
+        const long long t = t0 + (tid >> 6);
+        if (t < P.ntiles) {
+            const TileInfo ti = P.tiles[t];
+            const int x = ti.x0 + (tid & 7), y = ti.y0 + ((tid >> 3) & 7);
+            if ((ti.flags & 1) && x < nx && y < ny) {
+                const int m = P.midx[((long long)ti.z * ny + y) * nx + x];
+                if (m >= 0) nrow = nmo + ((long long)m * G + g0) * N;
+            }
+        }
+    }
+    const float *Ig = I + (ROWS ? 0 : (long long)g0 * P.Nc);
+    const long long kstride = (long long)G * P.Nc;
+    const bool rvec = (N & 3) == 0;
+    float4 pre[4];  // ROWS: the next chunk's pieces
+    auto load_rows = [&](int ch) {
 #pragma unroll
-            for (int i = 0; i < TR; ++i)
+        for (int i = 0; i < 4; ++i) {
+            const int r = (i & 1) * 64 + (tid >> 1), k = ch * KC + 8 * (i >> 1) + 4 * (tid & 1);
+            pre[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (row0 + r >= nrows || k >= N) continue;
+            const float *src = I + (row0 + r) * N + k;
+            if (rvec) {
+                pre[i] = *reinterpret_cast<const float4 *>(src);
+            } else {
+                pre[i].x = src[0];
+                if (k + 1 < N) pre[i].y = src[1];
+                if (k + 2 < N) pre[i].z = src[2];
+                if (k + 3 < N) pre[i].w = src[3];
+            }
+        }
+    };
+    auto put_rows = [&](int ch) {
+        float *A = As + (ch % kPStages) * KC * kPRow;
 #pragma unroll
-                for (int j = 0; j < TC; ++j) acc[i][j] = 0.f;
-            auto load_chunk = [&](int ch, int buf) {
-                float *A = As + (size_t)buf * KC * R;
-                for (int e = tid; e < KC * R; e += 256) {
-                    int kk = e >> 6, q = e & 63, k = ch * KC + kk;
-                    int r = q;
-                    bool ok = false;
-                    const float *src = nullptr;
-                    if (k < N) {
-                        int d = P.ord[k].d;
-                        r = tile_row(d, q);
-                        int ix = ti.x0 + (r & 7), iy = ti.y0 + (r >> 3);
-                        if (ix < P.nx && iy < P.ny) {
-                            const int m = P.midx[((long long)ti.z * P.ny + iy) * P.nx + ix];
-                            if (pass == 1 && m >= 0)
-                                src = I0 + ((long long)m * G + g) * N + k;  // comoving, node-major
-                            else
-                                src = I + ((long long)k * G + g) * P.Nc + perm_offset(d, ix, iy, ti.z, P.nx, P.ny, P.nz);
-                            ok = true;
-                        }
-                    }
-                    if (ok) cp_async4(&A[kk * R + r], src);
-                    else A[kk * R + r] = 0.f;
+        for (int i = 0; i < 4; ++i) {
+            const int r = (i & 1) * 64 + (tid >> 1), kk = 8 * (i >> 1) + 4 * (tid & 1);
+            A[kk * kPRow + r] = pre[i].x;
+            A[(kk + 1) * kPRow + r] = pre[i].y;
+            A[(kk + 2) * kPRow + r] = pre[i].z;
+            A[(kk + 3) * kPRow + r] = pre[i].w;
+        }
+    };
+    auto issue = [&](int ch) {
+        if (ch < nchunk) {
+            const int st = ch % kPStages;
+            float *B = Bs + st * KC * NBC;
+            for (int e = tid; e < KC * NBC / 4; e += 128) {
+                const int kk = e / (NBC / 4), c4 = e - kk * (NBC / 4), k = ch * KC + kk;
+                cp_async16(B + kk * NBC + 4 * c4, P.Bproj + (size_t)(k < N ? k : 0) * P.NB + 4 * c4, k < N);
+            }
+            if constexpr (!ROWS) {
+                float *A = As + st * KC * kPRow;
+#pragma unroll
+                for (int i = 0; i < (VEC ? 4 : 16); ++i) {
+                    const int kk = VEC ? (tid >> 5) + 4 * i : i, k = ch * KC + kk;
+                    const bool xc = k >= nA;
+                    const long long o = xc ? ox : (P.ord[k < N ? k : 0].d == 2 ? oz : oy);
+                    const bool on = k < N && (xc ? inx : inz);
+                    const float *src = on ? Ig + k * kstride + o : I;
+                    if constexpr (VEC) cp_async16(A + kk * kPRow + 4 * (tid & 31), src, on);
+                    else cp_async4(A + kk * kPRow + tid, src, on);
                 }
-                cp_async_commit();
-            };
-            __syncthreads();  // previous item's readers of As are done (and Bs is loaded)
-            load_chunk(0, 0);
-            for (int ch = 0; ch < nchunk; ++ch) {
-                if (ch + 1 < nchunk) {
-                    load_chunk(ch + 1, (ch + 1) & 1);
-                    cp_async_wait<1>();
+            }
+        }
+        cp_async_commit();
+    };
+
+    float acc[16][TN];
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
+    if constexpr (ROWS != 0) {
+        load_rows(0);
+        put_rows(0);
+        load_rows(1);
+    }
+    issue(0);
+    issue(1);
+    for (int ch = 0; ch < nchunk; ++ch) {
+        cp_async_wait<1>();
+        __syncthreads();  // chunk ch is visible; chunk ch - 1's readers are done
+        issue(ch + 2);
+        if constexpr (ROWS != 0) {
+            put_rows(ch + 1);
+            load_rows(ch + 2);
+        }
+        const float *A = As + (ch % kPStages) * KC * kPRow, *B = Bs + (ch % kPStages) * KC * NBC + tc;
+        const int kv = ROWS ? KC : (nA - ch * KC < KC ? (nA - ch * KC > 0 ? nA - ch * KC : 0) : KC);
+        if (!ROWS && nrow) {
+            const float *An = A + tid, *At = A + (tid & 64) + ((tid & 7) << 3) + ((tid >> 3) & 7);
+            float *dst = nrow + ch * KC;
+#pragma unroll
+            for (int q = 0; q < KC; q += 4) {
+                float v[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] = (q + e < kv ? An : At)[(q + e) * kPRow];
+                if (rvec) {
+                    if (ch * KC + q < N) *reinterpret_cast<float4 *>(dst + q) = make_float4(v[0], v[1], v[2], v[3]);
                 } else {
-                    cp_async_wait<0>();
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (ch * KC + q + e < N) dst[q + e] = v[e];
                 }
-                __syncthreads();
-                const float *A = As + (size_t)(ch & 1) * KC * R;
-                const int kbase = ch * KC;
-                const int kmax = N - kbase < KC ? N - kbase : KC;
-                if (tc * TC < ncol) {
-                    for (int kk = 0; kk < kmax; ++kk) {
-                        float4 a4 = *reinterpret_cast<const float4 *>(&A[kk * R + tr * TR]);
-                        const float *b = &Bs[(size_t)(kbase + kk) * NB + tc * TC];
-                        float bv[TC];
+            }
+        }
+#pragma unroll 2
+        for (int kk = 0; kk < kv; ++kk) {
+            float a[16], b[TN];
 #pragma unroll
-                        for (int j = 0; j < TC; ++j) bv[j] = b[j];
-                        float av[4] = {a4.x, a4.y, a4.z, a4.w};
-#pragma unroll
-                        for (int i = 0; i < TR; ++i)
-#pragma unroll
-                            for (int j = 0; j < TC; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-                    }
-                }
-                __syncthreads();  // buffer (ch & 1) may be refilled next
+            for (int q = 0; q < 4; ++q) {
+                const float4 v = *reinterpret_cast<const float4 *>(A + kk * kPRow + tr * 16 + 4 * q);
+                a[4 * q] = v.x; a[4 * q + 1] = v.y; a[4 * q + 2] = v.z; a[4 * q + 3] = v.w;
             }
 #pragma unroll
-            for (int i = 0; i < TR; ++i) {
-                int r = tr * TR + i;
-                int ix = ti.x0 + (r & 7), iy = ti.y0 + (r >> 3);
-                if (ix >= P.nx || iy >= P.ny) continue;
-                long long c = ((long long)ti.z * P.ny + iy) * P.nx + ix;
-                bool moving = P.mflag[c] != 0;
+            for (int j = 0; j < TN; ++j) b[j] = B[kk * NBC + 16 * j];
 #pragma unroll
-                for (int j = 0; j < TC; ++j) {
-                    int col = tc * TC + j;
-                    if (col < NLM) {
-                        if ((pass == 0 && !moving) || (pass == 1 && moving)) Ip[(c * G + g) * NLM + col] = acc[i][j];
-                    } else if (col < NLM + 10 && pass == 0) {
-                        mom[(c * G + g) * 10 + (col - NLM)] = acc[i][j];
-                    }
+            for (int i = 0; i < 16; ++i)
+#pragma unroll
+                for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+        }
+        if constexpr (!ROWS) {
+#pragma unroll 2
+            for (int kk = kv; kk < KC; ++kk) {
+                float a[16], b[TN];
+                const float *At = A + kk * kPRow + (tr >> 2) * 64 + 2 * (tr & 3);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const float2 v = *reinterpret_cast<const float2 *>(At + 8 * i);
+                    a[i] = v.x;
+                    a[8 + i] = v.y;
                 }
+#pragma unroll
+                for (int j = 0; j < TN; ++j) b[j] = B[kk * NBC + 16 * j];
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+#pragma unroll
+                    for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+            }
+        }
+    }
+    cp_async_wait<0>();
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        long long cg;
+        bool sh = true;
+        if constexpr (ROWS != 0) {
+            const long long row = row0 + tr * 16 + i;
+            if (row >= nrows) break;
+            const long long m = row / G;
+            cg = P.moving[m] * G + (row - m * G);
+        } else {
+            const long long t = t0 + (tr >> 2);
+            if (t >= P.ntiles) break;
+            const TileInfo ti = P.tiles[t];
+            const int x = ti.x0 + (i & 7), y = ti.y0 + 2 * (tr & 3) + (i >> 3);
+            if (x >= nx || y >= ny) continue;
+            const long long c = ((long long)ti.z * ny + y) * nx + x;
+            cg = c * G + g0;
+            sh = P.mflag[c] == 0;
+        }
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+            const int col = tc + 16 * j;
+            if (col < NLM) {
+                if (sh) Ip[cg * NLM + col] = acc[i][j];
+            } else if (!ROWS && col < NLM + 10) {
+                mom[cg * 10 + (col - NLM)] = acc[i][j];
             }
         }
     }
 }
 
-// a3, persistent: Bs = Y^T [NLM][N] resident; per item As [NLM][64], the
-// result staged per 128-ordinate chunk in Cs [128][65] and written as runs.
-__global__ void __launch_bounds__(256, 1) k_sh2lab_persist(Prob<float> P, const float *__restrict__ Sp,
-                                                           float *__restrict__ eta, float *__restrict__ chi,
-                                                           float *__restrict__ S0)
+// a3: [64 nodes x NLM] x [NLM x ordinates] per (brick, group).  A CTA is
+// persistent over the (brick, group) items for one slice of the ordinates,
+// at most kSGroups groups of 16 of one kind (z- and y-class, or x-class),
+// with that slice of Y^T resident in shared memory; three CTAs share an SM,
+// so one's stores and barriers overlap another's FMAs (one CTA for all
+// ordinates spent 40 % of its time at its barriers).  A thread computes four
+// nodes of a run (along x; for x-class slices along y, S staged transposed) x
+// the 16 ordinates of a group: 16 threads a group, lanes pairwise completing
+// 32-byte runs.  S is staged as it lies, rows of harmonics, by cp.async one
+// item ahead; 16-byte pieces are swizzled by the row so that a thread's four
+// harmonics of a node are one conflict-free 16-byte load.  ROWS = 1 covers
+// the bricks that hold a moving node and stores those nodes' comoving S0
+// node-major for their remap (k_nodes_to_brick brings the result back; read
+// here instead, it cost this kernel 3.8 ms for the pass's 2.2); ROWS = 0
+// stores eta of nodes at rest, and chi where it is not the kept chi0
+// (chi_all), or in a run of four that holds a moving node.
+constexpr int kSGroups = 9, kSThreads = 160;
+
+// slices of the z- and y-class groups (nA ordinates), of the x-class groups,
+// and groups a slice
+struct SliceShape {
+    int nsA, nsX, gA, gX;
+};
+__host__ __device__ inline SliceShape sh2lab_f32_slices(int nA, int N)
 {
-    constexpr int R = 64, KC = 128, TR = 8, TC = 4;
+    SliceShape h;
+    const int a = (nA + 15) / 16, x = (N - nA + 15) / 16;
+    h.nsA = (a + kSGroups - 1) / kSGroups;
+    h.nsX = (x + kSGroups - 1) / kSGroups;
+    h.gA = h.nsA ? (a + h.nsA - 1) / h.nsA : 0;
+    h.gX = h.nsX ? (x + h.nsX - 1) / h.nsX : 0;
+    return h;
+}
+
+template <int ROWS>
+__global__ void __launch_bounds__(kSThreads, 3) k_sh2lab_f32(Prob<float> P, const float *__restrict__ Sp,
+                                                             float *__restrict__ eta, float *__restrict__ chi,
+                                                             float *__restrict__ S0, int nZ, int nA, int chi_all)
+{
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int NLM = P.NLM, N = P.N, G = P.G;
-    float *Bs = reinterpret_cast<float *>(smem_raw);  // [NLM][N]
-    float *As = Bs + (size_t)NLM * N;                  // [NLM][R]
-    float *Cs = As + (size_t)NLM * R;                  // [KC][R + 1]
-    float *chir = Cs + (size_t)KC * (R + 1);           // [R]
-    int *mrow = reinterpret_cast<int *>(chir + R);     // [R] moving index, -1 at rest
-    const int tid = threadIdx.x, tr = tid >> 5, tc = tid & 31;
-    for (int e = tid; e < N * NLM; e += 256) {
-        int k = e / NLM, p = e - k * NLM;
-        Bs[(size_t)p * N + k] = P.Y[e];
+    const int NLM = P.NLM, N = P.N, G = P.G, nx = P.nx, ny = P.ny, nz = P.nz;
+    const SliceShape sh = sh2lab_f32_slices(nA, N);
+    const int nsl = sh.nsA + sh.nsX, sl = (int)(blockIdx.x % nsl);
+    const bool xc = sl >= sh.nsA;
+    const int gs = xc ? sh.gX : sh.gA, NS = gs * 16;
+    const int kb = xc ? nA + (sl - sh.nsA) * NS : sl * NS;                          // the slice's first ordinate
+    const int kend = xc ? N : (kb + NS < nA ? kb + NS : nA);                        // and its end
+    const int smax = (sh.gA > sh.gX ? sh.gA : sh.gX) * 16;
+    float *Bs = reinterpret_cast<float *>(smem_raw);  // [NLM][NS]
+    const int NP = (NLM + 3) & ~3, pitch = (NLM + 31) & ~31;
+    float *As = Bs + (size_t)NP * smax;                // [2 items][64][pitch]
+    float *chir = As + (size_t)2 * 64 * pitch;         // [2][64], rows of the brick in staged order
+    int *mrow = reinterpret_cast<int *>(chir + 128);   // [2][64]: moving index, -1 at rest, -2 outside
+    const int tid = threadIdx.x, nthr = blockDim.x;
+    for (int e = tid; e < NP * NS; e += nthr) {
+        const int q = e / NP, p = e - q * NP;
+        Bs[p * NS + q] = kb + q < kend && p < NLM ? P.Y[(size_t)(kb + q) * NLM + p] : 0.f;
     }
-    const long long items = P.ntiles * G;
-    for (long long w = blockIdx.x; w < items; w += gridDim.x) {
-        const long long tile = w / G;
-        const int g = (int)(w - tile * G);
-        const TileInfo ti = P.tiles[tile];
-        __syncthreads();
-        for (int e = tid; e < R * NLM; e += 256) {
-            int r = e / NLM, p = e - r * NLM;
-            int ix = ti.x0 + (r & 7), iy = ti.y0 + (r >> 3);
-            float v = 0.f;
-            if (ix < P.nx && iy < P.ny) {
-                long long c = ((long long)ti.z * P.ny + iy) * P.nx + ix;
-                v = Sp[(c * G + g) * NLM + p];
+    for (int e = tid; e < 2 * 64 * pitch; e += nthr) As[e] = 0.f;  // rows outside the grid and the padding stay zero
+    __syncthreads();
+    const int nt = (int)(ROWS ? P.nmtiles : P.ntiles);
+    const long long items = (long long)nt * G;
+    // node of staged row r: z- and y-class along x, x-class along y
+    auto row_xy = [&](const TileInfo &ti, int r, int &x, int &y) {
+        x = ti.x0 + (xc ? r >> 3 : r & 7);
+        y = ti.y0 + (xc ? r & 7 : r >> 3);
+        return x < nx && y < ny;
+    };
+    // 16-byte piece c of row r
+    auto piece = [](int r, int c) { return (c & ~7) | ((c ^ (r >> 2)) & 7); };
+    // items in order of (group, tile): w = g nt + t
+    struct Item {
+        TileInfo ti;
+        int g;
+    };
+    auto item_of = [&](long long w) {
+        Item it;
+        it.g = (int)(w / nt);
+        const int t = (int)(w - (long long)it.g * nt);
+        it.ti = P.tiles[ROWS ? P.mtiles[t] : t];
+        return it;
+    };
+    float pch = 0.f;
+    int pm = -2;
+    auto load_item = [&](const Item &it, int b) {
+        float *A = As + b * 64 * pitch;
+        int x, y;
+        if ((NLM & 3) == 0) {
+            const int np = NLM >> 2;
+            for (int e = tid; e < 64 * np; e += nthr) {
+                const int r = e / np, c = e - r * np;
+                const bool on = row_xy(it.ti, r, x, y);
+                const float *src = on ? Sp + ((((long long)it.ti.z * ny + y) * nx + x) * G + it.g) * NLM + 4 * c : Sp;
+                cp_async16(A + r * pitch + 4 * piece(r, c), src, on);
             }
-            As[(size_t)p * R + r] = v;
-        }
-        for (int r = tid; r < R; r += 256) {
-            int ix = ti.x0 + (r & 7), iy = ti.y0 + (r >> 3);
-            float ch = 0.f;
-            int m = -1;
-            if (ix < P.nx && iy < P.ny) {
-                long long c = ((long long)ti.z * P.ny + iy) * P.nx + ix;
-                ch = P.chi0[c * G + g];
-                m = P.midx[c];
+        } else {
+            for (int e = tid; e < 64 * NLM; e += nthr) {
+                const int r = e / NLM, p = e - r * NLM;
+                const bool on = row_xy(it.ti, r, x, y);
+                const float *src = on ? Sp + ((((long long)it.ti.z * ny + y) * nx + x) * G + it.g) * NLM + p : Sp;
+                cp_async4(A + r * pitch + 4 * piece(r, p >> 2) + (p & 3), src, on);
             }
-            chir[r] = ch;
-            mrow[r] = m;
         }
-        __syncthreads();
-        for (int k0 = 0; k0 < N; k0 += KC) {
-            float acc[TR][TC];
+        cp_async_commit();
+        pm = -2;
+        if (tid < 64 && row_xy(it.ti, tid, x, y)) {
+            const long long c = ((long long)it.ti.z * ny + y) * nx + x;
+            pch = P.chi0[c * G + it.g];
+            pm = P.midx[c];
+        }
+    };
+    auto put_item = [&](int b) {
+        cp_async_wait<0>();
+        if (tid < 64) {
+            chir[b * 64 + tid] = pch;
+            mrow[b * 64 + tid] = pm;
+        }
+    };
+    const int j = (tid >> 1) & 7, h4 = 4 * (tid & 1), r0 = j * 8 + h4;  // staged rows r0 .. r0 + 3
+    const bool rows16 = (nx & 3) == 0 && (ny & 3) == 0;                 // runs of four nodes are 16-byte aligned
+    const bool kvec = (N & 3) == 0;
+    const long long w0 = blockIdx.x / nsl, ws = gridDim.x / nsl;
+    Item cur, nxt;
+    if (w0 < items) {
+        cur = item_of(w0);
+        load_item(cur, 0);
+        put_item(0);
+    }
+    int buf = 0;
+    for (long long w = w0; w < items; w += ws, buf ^= 1) {
+        __syncthreads();  // this item's S is in place; the other buffer's readers are done
+        const bool more = w + ws < items;
+        if (more) {
+            nxt = item_of(w + ws);
+            load_item(nxt, buf ^ 1);
+        }
+        const int gr = tid >> 4;
+        if (gr < gs && kb + gr * 16 < kend) {
+            const float *A = As + (buf * 64 + r0) * pitch;
+            const float *B = Bs + gr * 16;
+            float acc[4][16];
 #pragma unroll
-            for (int i = 0; i < TR; ++i)
+            for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int j = 0; j < TC; ++j) acc[i][j] = 0.f;
-            for (int p = 0; p < NLM; ++p) {
-                const float *a = &As[(size_t)p * R + tr * TR];
-                float4 a0 = *reinterpret_cast<const float4 *>(a);
-                float4 a1 = *reinterpret_cast<const float4 *>(a + 4);
-                float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-                float bv[TC];
+                for (int q = 0; q < 16; ++q) acc[i][q] = 0.f;
+            for (int c = 0; c < NP / 4; ++c) {
+                float a[4][4];  // [node][harmonic]
 #pragma unroll
-                for (int j = 0; j < TC; ++j) {
-                    int k = k0 + tc + 32 * j;
-                    bv[j] = k < N ? Bs[(size_t)p * N + k] : 0.f;
+                for (int i = 0; i < 4; ++i) {
+                    const float4 v = *reinterpret_cast<const float4 *>(A + i * pitch + 4 * piece(r0, c));
+                    a[i][0] = v.x; a[i][1] = v.y; a[i][2] = v.z; a[i][3] = v.w;
                 }
 #pragma unroll
-                for (int i = 0; i < TR; ++i)
+                for (int pp = 0; pp < 4; ++pp)
 #pragma unroll
-                    for (int j = 0; j < TC; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+                    for (int q4 = 0; q4 < 4; ++q4) {
+                        const float4 b = *reinterpret_cast<const float4 *>(B + (4 * c + pp) * NS + 4 * q4);
+                        const float bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+#pragma unroll
+                            for (int q = 0; q < 4; ++q)
+                                acc[i][4 * q4 + q] = fmaf(a[i][pp], bv[q], acc[i][4 * q4 + q]);
+                    }
             }
+            const int k0 = kb + gr * 16, kn = kend - k0 < 16 ? kend - k0 : 16;
+            float ch[4];
+            int m[4];
+            bool rest = true, moves = false;
 #pragma unroll
-            for (int i = 0; i < TR; ++i)
+            for (int i = 0; i < 4; ++i) {
+                ch[i] = chir[buf * 64 + r0 + i];
+                m[i] = mrow[buf * 64 + r0 + i];
+                rest = rest && m[i] == -1;
+                moves = moves || m[i] >= 0;
+            }
+            const bool vec = kvec && kn == 16 && (k0 & 3) == 0;
+            if constexpr (ROWS != 0) {
 #pragma unroll
-                for (int j = 0; j < TC; ++j) Cs[(size_t)(tc + 32 * j) * (R + 1) + tr * TR + i] = acc[i][j];
-            __syncthreads();
-            for (int e = tid; e < KC * R; e += 256) {
-                int kk = e >> 6, q = e & 63, k = k0 + kk;
-                if (k >= N) continue;
-                int d = P.ord[k].d;
-                int r = tile_row(d, q);
-                int ix = ti.x0 + (r & 7), iy = ti.y0 + (r >> 3);
-                if (ix >= P.nx || iy >= P.ny) continue;
-                float v = Cs[(size_t)kk * (R + 1) + r];
-                const int m = mrow[r];
-                if (m >= 0) {
-                    S0[((long long)m * G + g) * N + k] = v;  // comoving, node-major
-                } else {
-                    long long a = ((long long)k * G + g) * P.Nc + perm_offset(d, ix, iy, ti.z, P.nx, P.ny, P.nz);
-                    float ch = chir[r];
-                    eta[a] = ch * v;
-                    chi[a] = ch;
+                for (int i = 0; i < 4; ++i) {
+                    if (m[i] < 0) continue;
+                    float *dst = S0 + ((long long)m[i] * G + cur.g) * N + k0;
+                    if (vec) {
+#pragma unroll
+                        for (int q4 = 0; q4 < 4; ++q4)
+                            reinterpret_cast<float4 *>(dst)[q4] =
+                                make_float4(acc[i][4 * q4], acc[i][4 * q4 + 1], acc[i][4 * q4 + 2], acc[i][4 * q4 + 3]);
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < 16; ++q)
+                            if (q < kn) dst[q] = acc[i][q];
+                    }
+                }
+            } else {
+                const bool wchi = chi_all || moves;
+                const int x = cur.ti.x0 + (xc ? j : h4), y = cur.ti.y0 + (xc ? h4 : j);
+                const long long oz = ((long long)cur.ti.z * ny + y) * nx + x, oy = ((long long)y * nz + cur.ti.z) * nx + x;
+                const long long ox = ((long long)x * nz + cur.ti.z) * ny + y;
+                const long long kst = (long long)G * P.Nc;
+                const long long og = (long long)k0 * kst + (long long)cur.g * P.Nc;
+#pragma unroll
+                for (int q = 0; q < 16; ++q) {
+                    if (q >= kn) break;
+                    const long long o = og + q * kst + (xc ? ox : (k0 + q < nZ ? oz : oy));
+                    if (rest && rows16) {
+                        *reinterpret_cast<float4 *>(eta + o) =
+                            make_float4(ch[0] * acc[0][q], ch[1] * acc[1][q], ch[2] * acc[2][q], ch[3] * acc[3][q]);
+                        if (wchi) *reinterpret_cast<float4 *>(chi + o) = make_float4(ch[0], ch[1], ch[2], ch[3]);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            if (m[i] != -1) continue;
+                            eta[o + i] = ch[i] * acc[i][q];
+                            if (wchi) chi[o + i] = ch[i];
+                        }
+                    }
                 }
             }
-            __syncthreads();
+        }
+        if (more) {
+            put_item(buf ^ 1);
+            cur = nxt;
         }
     }
 }
@@ -1069,45 +1327,98 @@ static int num_sms(const shd_ctx *ctx)
 
 static const size_t kSmemLimit = 227 * 1024;
 
-size_t project_persist_smem_bytes(const shd_ctx *c)
-{
-    return sizeof(float) * ((size_t)c->N * c->NB + 2 * 32 * 64);
-}
-size_t sh2lab_persist_smem_bytes(const shd_ctx *c)
-{
-    return sizeof(float) * ((size_t)c->NLM * c->N + (size_t)c->NLM * 64 + 128 * 65 + 64) + 64 * 4 + 64;
-}
+// rows of the grid along x and y are 16-byte multiples
+static bool rows_aligned(const shd_ctx *c) { return c->nx % 4 == 0 && c->ny % 4 == 0; }
 
-template <int TC>
-static cudaError_t launch_project_persist_tc(const shd_ctx *ctx, const float *I, float *Ip, float *mom,
-                                             const float *scratch, cudaStream_t st)
+template <int TN, int ROWS, bool VEC>
+static cudaError_t launch_project_f32_k(const shd_ctx *ctx, const float *I, float *Ip, float *mom, float *nmo,
+                                        cudaStream_t st)
 {
-    Prob<float> P = make_prob<float>(ctx);
-    size_t sm = project_persist_smem_bytes(ctx);
-    cudaError_t e = cudaFuncSetAttribute(k_project_persist<TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const Prob<float> P = make_prob<float>(ctx);
+    const int sm = (int)sizeof(float) * kPStages * kPKC * (kPRow + 16 * TN);
+    auto kern = k_project_f32<TN, ROWS, VEC>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     if (e != cudaSuccess) return e;
-    long long items = ctx->ntiles * ctx->G;
-    int grid = num_sms(ctx);
-    if (items < grid) grid = (int)items;
-    k_project_persist<TC><<<grid, 256, sm, st>>>(P, I, scratch, Ip, mom);
+    const long long ntp = (ctx->ntiles + 1) / 2;
+    const long long grid = ROWS ? (ctx->nmoving * ctx->G + 127) / 128 : ntp * ctx->G;
+    kern<<<(unsigned)grid, 128, sm, st>>>(P, I, Ip, mom, nmo, ctx->nA, ntp);
     note_launch();
     return cudaGetLastError();
 }
 
-static cudaError_t launch_project_persist(const shd_ctx *ctx, const float *I, float *Ip, float *mom,
-                                          const float *scratch, cudaStream_t st)
+template <int ROWS, bool VEC>
+static cudaError_t launch_project_f32_tn(const shd_ctx *ctx, int tn, const float *I, float *Ip, float *mom,
+                                         float *nmo, cudaStream_t st)
 {
-    switch (ctx->NB / 16) {
-        case 1: return launch_project_persist_tc<1>(ctx, I, Ip, mom, scratch, st);
-        case 2: return launch_project_persist_tc<2>(ctx, I, Ip, mom, scratch, st);
-        case 3: return launch_project_persist_tc<3>(ctx, I, Ip, mom, scratch, st);
-        case 4: return launch_project_persist_tc<4>(ctx, I, Ip, mom, scratch, st);
-        case 5: return launch_project_persist_tc<5>(ctx, I, Ip, mom, scratch, st);
-        case 6: return launch_project_persist_tc<6>(ctx, I, Ip, mom, scratch, st);
-        case 7: return launch_project_persist_tc<7>(ctx, I, Ip, mom, scratch, st);
-        case 8: return launch_project_persist_tc<8>(ctx, I, Ip, mom, scratch, st);
+    switch (tn) {
+        case 1: return launch_project_f32_k<1, ROWS, VEC>(ctx, I, Ip, mom, nmo, st);
+        case 2: return launch_project_f32_k<2, ROWS, VEC>(ctx, I, Ip, mom, nmo, st);
+        case 3: return launch_project_f32_k<3, ROWS, VEC>(ctx, I, Ip, mom, nmo, st);
+        case 4: return launch_project_f32_k<4, ROWS, VEC>(ctx, I, Ip, mom, nmo, st);
+        case 5: return launch_project_f32_k<5, ROWS, VEC>(ctx, I, Ip, mom, nmo, st);
+        case 6: return launch_project_f32_k<6, ROWS, VEC>(ctx, I, Ip, mom, nmo, st);
+        case 7: return launch_project_f32_k<7, ROWS, VEC>(ctx, I, Ip, mom, nmo, st);
+        case 8: return launch_project_f32_k<8, ROWS, VEC>(ctx, I, Ip, mom, nmo, st);
         default: return cudaErrorInvalidConfiguration;
     }
+}
+
+// the laboratory rows' columns [W Y | moments] and the moving rows' copy, then
+// the comoving remap and the moving rows' W Y
+static cudaError_t launch_project_f32(const shd_ctx *ctx, const float *I, float *Ip, float *mom, float *nm0,
+                                      float *nm1, cudaStream_t st)
+{
+    const int tn = ctx->NB / 16;
+    cudaError_t e = rows_aligned(ctx) ? launch_project_f32_tn<0, true>(ctx, tn, I, Ip, mom, nm0, st)
+                                      : launch_project_f32_tn<0, false>(ctx, tn, I, Ip, mom, nm0, st);
+    if (e != cudaSuccess || ctx->nmoving == 0) return e;
+    if ((e = launch_remap_to_comoving_f(ctx, nm0, nm1, st)) != cudaSuccess) return e;
+    return launch_project_f32_tn<1, true>(ctx, (ctx->NLM + 15) / 16, nm1, Ip, mom, nullptr, st);
+}
+
+static size_t sh2lab_f32_smem_bytes(const shd_ctx *c)
+{
+    const SliceShape h = sh2lab_f32_slices(c->nA, c->N);
+    return sizeof(float) * ((size_t)((c->NLM + 3) & ~3) * 16 * std::max(h.gA, h.gX) +
+                            (size_t)2 * 64 * ((c->NLM + 31) & ~31) + 256);
+}
+
+// FP32's a3 keeps chi_lab at rest (as the mixed segment transform does)
+bool sh2lab_f32_usable(const shd_ctx *c)
+{
+    return c->precision == SHD_FP32 && sh2lab_f32_smem_bytes(c) <= kSmemLimit;
+}
+
+template <int ROWS>
+static cudaError_t launch_sh2lab_f32_k(const shd_ctx *ctx, const float *Sp, float *eta, float *chi, float *S0,
+                                       cudaStream_t st, bool full_chi)
+{
+    const Prob<float> P = make_prob<float>(ctx);
+    const size_t sm = sh2lab_f32_smem_bytes(ctx);
+    auto kern = k_sh2lab_f32<ROWS>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    const long long items = (ROWS ? ctx->nmtiles : ctx->ntiles) * ctx->G;
+    const SliceShape h = sh2lab_f32_slices(ctx->nA, ctx->N);
+    const int nsl = h.nsA + h.nsX;
+    const int nthr = std::max(64, (16 * std::max(h.gA, h.gX) + 31) & ~31);
+    int per = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, nthr, sm) != cudaSuccess || per < 1) per = 1;
+    // every slice over as many CTAs
+    const long long ctas = std::min<long long>(items, std::max(1, num_sms(ctx) * per / nsl));
+    const long long grid = ctas * nsl;
+    kern<<<(unsigned)grid, nthr, sm, st>>>(P, Sp, eta, chi, S0, ctx->nZ, ctx->nA, full_chi ? 1 : 0);
+    note_launch();
+    return cudaGetLastError();
+}
+
+// eta and chi of nodes at rest, S0 of moving nodes
+static cudaError_t launch_sh2lab_f32(const shd_ctx *ctx, const float *Sp, float *eta, float *chi, float *S0,
+                                     cudaStream_t st, bool full_chi)
+{
+    const cudaError_t e = launch_sh2lab_f32_k<0>(ctx, Sp, eta, chi, nullptr, st, full_chi);
+    if (e != cudaSuccess || ctx->nmoving == 0) return e;
+    return launch_sh2lab_f32_k<1>(ctx, Sp, nullptr, nullptr, S0, st, false);
 }
 
 template <class T>
@@ -1168,6 +1479,7 @@ cudaError_t launch_project_nm(const shd_ctx *ctx, const T *I, T *Ip, T *mom, T *
     if constexpr (sizeof(T) == 4) {
         // the segment kernels write the moving rows node-major themselves
         if (seg_usable(ctx)) return launch_project_seg(ctx, I, Ip, mom, nm0, nm1, st);
+        if (!tc_usable(ctx)) return launch_project_f32(ctx, I, Ip, mom, nm0, nm1, st);
     }
     if (ctx->nmoving > 0) {
         k_brick_to_nodes<T><<<(unsigned)(ctx->nmtiles * ctx->G), 256, 0, st>>>(P, I, nm0);
@@ -1175,11 +1487,8 @@ cudaError_t launch_project_nm(const shd_ctx *ctx, const T *I, T *Ip, T *mom, T *
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         if ((e = run_remap_to_comoving<T>(ctx, nm0, nm1, st)) != cudaSuccess) return e;
     }
-    if constexpr (sizeof(T) == 4) {
-        if (tc_usable(ctx)) return launch_project_tc(ctx, I, Ip, mom, nm1, st);
-        if (project_persist_smem_bytes(ctx) <= kSmemLimit) return launch_project_persist(ctx, I, Ip, mom, nm1, st);
-    }
-    switch (ctx->NB / 16) {
+    if constexpr (sizeof(T) == 4) return launch_project_tc(ctx, I, Ip, mom, nm1, st);
+    else switch (ctx->NB / 16) {
         case 1: return launch_project_tile_tc<T, 1>(ctx, I, nm1, Ip, mom, st);
         case 2: return launch_project_tile_tc<T, 2>(ctx, I, nm1, Ip, mom, st);
         case 3: return launch_project_tile_tc<T, 3>(ctx, I, nm1, Ip, mom, st);
@@ -1208,21 +1517,14 @@ cudaError_t launch_sh2lab(const shd_ctx *ctx, const T *Sp, T *eta, T *chi, cudaS
     T *nm0 = (T *)ctx->d_nm[0], *nm1 = (T *)ctx->d_nm[1], *nm2 = (T *)ctx->d_nm[2];
     bool done = false;
     if constexpr (sizeof(T) == 4) {
-        size_t smp = sh2lab_persist_smem_bytes(ctx);
         // the segment kernels run the remap and write the moving rows themselves
         if (seg_usable(ctx)) return launch_sh2lab_seg(ctx, Sp, eta, chi, nm0, nm1, nm2, st, full_chi);
         if (tc_usable(ctx)) {
             if ((e = launch_sh2lab_tc(ctx, Sp, eta, chi, nm0, st)) != cudaSuccess) return e;
             done = true;
-        } else if (smp <= kSmemLimit) {
-            e = cudaFuncSetAttribute(k_sh2lab_persist, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smp);
-            if (e != cudaSuccess) return e;
-            long long items = ctx->ntiles * ctx->G;
-            int grid = num_sms(ctx);
-            if (items < grid) grid = (int)items;
-            k_sh2lab_persist<<<grid, 256, smp, st>>>(P, Sp, eta, chi, nm0);
-            note_launch();
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        } else if (sh2lab_f32_smem_bytes(ctx) <= kSmemLimit) {
+            if ((e = launch_sh2lab_f32(ctx, Sp, eta, chi, nm0, st, full_chi || !sh2lab_f32_usable(ctx))) != cudaSuccess)
+                return e;
             done = true;
         }
     }
