@@ -660,7 +660,8 @@ template <class T>
 int set_state_impl(shd_ctx *c, const double *src, bool host, cudaStream_t st, T *dst)
 {
     size_t per_node = (size_t)c->G * c->N;
-    long long chunk = (long long)(c->stage_elems / per_node);
+    // host data passes through the staging buffer, device data in one piece
+    long long chunk = host ? (long long)(c->stage_elems / per_node) : c->Nc;
     if (chunk < 1) chunk = 1;
     for (long long c0 = 0; c0 < c->Nc; c0 += chunk) {
         long long nc = c->Nc - c0 < chunk ? c->Nc - c0 : chunk;
@@ -678,7 +679,7 @@ template <class T>
 int get_state_impl(shd_ctx *c, const T *src, double *dst, bool host, cudaStream_t st)
 {
     size_t per_node = (size_t)c->G * c->N;
-    long long chunk = (long long)(c->stage_elems / per_node);
+    long long chunk = host ? (long long)(c->stage_elems / per_node) : c->Nc;
     if (chunk < 1) chunk = 1;
     for (long long c0 = 0; c0 < c->Nc; c0 += chunk) {
         long long nc = c->Nc - c0 < chunk ? c->Nc - c0 : chunk;
@@ -991,7 +992,6 @@ int step_full(shd_ctx *c, cudaStream_t st)
     T *I = (T *)c->d_I, *A = (T *)c->d_rk[0], *B = (T *)c->d_rk[1], *acc = (T *)c->d_rk[2];
     if (!A || !B || !acc || !c->d_sums_save) return fail(SHD_ERR_STATE, "Runge-Kutta arrays missing");
     CK(cudaMemcpyAsync(A, I, n * sizeof(T), cudaMemcpyDeviceToDevice, st), "RK copy");
-    CK(cudaMemcpyAsync(B, I, n * sizeof(T), cudaMemcpyDeviceToDevice, st), "RK copy");
     static const double frac[4] = {1.0 / 6.0, 1.0 / 3.0, 1.0 / 3.0, 1.0 / 6.0};
     static const double cnext[4] = {3.0, 1.5, 3.0, 0.0};
     const double kap = c->kappa;
@@ -1004,7 +1004,7 @@ int step_full(shd_ctx *c, cudaStream_t st)
             cudaError_t e = cudaMemcpyAsync(c->d_sums_save, c->d_sums, 2 * sizeof(double), cudaMemcpyDeviceToDevice, st);
             if (e != cudaSuccess) { rc = cuda_fail(e, "save sums"); break; }
         }
-        cudaError_t e = launch_rk_stage<T>(I, A, B, acc, n, cnext[i], i == 0, i == 3, st);
+        cudaError_t e = launch_rk_stage<T>(I, A, B, acc, n, cnext[i], i, st);
         if (e != cudaSuccess) { rc = cuda_fail(e, "Runge-Kutta stage"); break; }
         if (i < 3) {
             std::swap(c->d_Sp, c->d_Sprev);

@@ -11,6 +11,7 @@
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -916,7 +917,7 @@ __global__ void k_sums_partial(Prob<T> P, const T *__restrict__ mom, const T *__
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nJ; i += stride) {
         int g = (int)(i % P.G);
         double J = (double)mom[i * 10];
-        double de = P.edges[g + 1] - P.edges[g];
+        const double de = P.edges[g + 1] - P.edges[g];
         e += 4.0 * kPi * J * de;
         ph += 4.0 * kPi * J * de / P.centre[g];
     }
@@ -1041,26 +1042,39 @@ __global__ void k_ng_combine(T *__restrict__ x0, const T *__restrict__ x1, const
 
 // -------------------------------------------------------------------------
 // Runge-Kutta sub-stepping of a time step (App. A, eq:rk4th).  A holds
-// I(t), B the input of the sub-solve just run, I its result; with
-// dI = I - B:  acc = dI (first) or acc + dI;  then either the next input
-// I = B = A + c dI, or (last) the new state I = A + acc.
+// I(t), I the result of the sub-solve just run; with dI = I - its input:
+// acc = dI (first) or acc + dI;  then either the next input I = A + c dI, or
+// (last) the new state I = A + acc.
 // -------------------------------------------------------------------------
-template <class T>
-__global__ void k_rk_stage(T *__restrict__ I, const T *__restrict__ A, T *__restrict__ B, T *__restrict__ acc,
-                           long long n, T cnext, int first, int last)
+// STAGE 0..3: the sub-solve just done.  Its input is I(t) = A after stage 0,
+// A + 3 acc (formed here again, as stage 0 formed it) after stage 1, B after
+// stages 2 and 3, so B is written by stages 1 and 2 only.  16 bytes a thread
+// and array (VEC; the arrays' tail by the scalar form): memory-bound, 24 array
+// passes a step where a copy of I(t) into B and a stored B for every stage
+// made 29 (3.39 ms on a 32^3, 16-group shell at L = 5 with the copies,
+// 2.0 now).
+template <class T, int STAGE, int V>
+__global__ void __launch_bounds__(256) k_rk_stage(T *__restrict__ I, const T *__restrict__ A, T *__restrict__ B,
+                                                  T *__restrict__ acc, long long i0, long long n, T cnext)
 {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const long long i = i0 + (blockIdx.x * (long long)blockDim.x + threadIdx.x) * V;
     if (i >= n) return;
-    const T d = I[i] - B[i];
-    const T s = first ? d : acc[i] + d;
-    if (last) {
-        I[i] = A[i] + s;
-        return;
+    struct alignas(V * sizeof(T)) Vec {
+        T v[V];
+    };
+    Vec y = *reinterpret_cast<const Vec *>(I + i), a = *reinterpret_cast<const Vec *>(A + i), s, x;
+    if constexpr (STAGE > 0) s = *reinterpret_cast<const Vec *>(acc + i);
+    if constexpr (STAGE > 1) x = *reinterpret_cast<const Vec *>(B + i);
+#pragma unroll
+    for (int j = 0; j < V; ++j) {
+        const T in = STAGE == 0 ? a.v[j] : (STAGE == 1 ? a.v[j] + T(3) * s.v[j] : x.v[j]);
+        const T d = y.v[j] - in;
+        s.v[j] = STAGE == 0 ? d : s.v[j] + d;
+        x.v[j] = STAGE == 3 ? a.v[j] + s.v[j] : a.v[j] + cnext * d;
     }
-    acc[i] = s;
-    const T x = A[i] + cnext * d;
-    I[i] = x;
-    B[i] = x;
+    *reinterpret_cast<Vec *>(I + i) = x;
+    if constexpr (STAGE < 3) *reinterpret_cast<Vec *>(acc + i) = s;
+    if constexpr (STAGE == 1 || STAGE == 2) *reinterpret_cast<Vec *>(B + i) = x;
 }
 
 // -------------------------------------------------------------------------
@@ -1450,40 +1464,87 @@ __global__ void __launch_bounds__(256) k_source_thermal(Prob<T> P, const T *__re
 // -------------------------------------------------------------------------
 // layout conversions
 // -------------------------------------------------------------------------
-template <class T>
-__global__ void k_canon_to_do(Prob<T> P, const double *__restrict__ src, T *__restrict__ dst, long long c0,
-                              long long nc)
+// Canonical FP64 [c][g][k] (mesh order) <-> the discrete-ordinate layout
+// [k][g][o], TO_DO or back: an 8 x 8 brick of nodes in one group per CTA, 32
+// mesh ordinates at a time through shared memory.  The canonical side moves
+// in 256-byte rows of ordinates, the other in 32-byte runs of nodes; a
+// thread's eight values of a chunk are in flight together.  One thread an
+// element, as this was, one of the two sides moved 4 bytes a 32-byte sector:
+// 32^3, 16 groups, 288 ordinates 2.00 and 1.93 ms, 0.74 and 0.71 now.
+// Nodes [c0, c0 + nc) only; canon points at node c0's values.
+template <class T, bool TO_DO>
+__global__ void __launch_bounds__(256) k_state_transpose(Prob<T> P, const double *__restrict__ canon_in,
+                                                         double *__restrict__ canon_out, T *__restrict__ dov,
+                                                         long long c0, long long nc, int z0, long long nbr)
 {
-    long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    const int G = P.G, N = P.N;
-    long long n = nc * G * N;
-    if (i >= n) return;
-    int k = (int)(i % N);
-    long long cg = i / N;
-    int g = (int)(cg % G);
-    long long c = c0 + cg / G;
-    int ix, iy, iz;
-    node_xyz(c, P.nx, P.ny, ix, iy, iz);
-    const int ki = P.mesh2int[k];  // canonical arrays are in mesh order
-    dst[((long long)ki * G + g) * P.Nc + perm_offset(P.ord[ki].d, ix, iy, iz, P.nx, P.ny, P.nz)] = (T)src[i];
-}
-
-template <class T>
-__global__ void k_do_to_canon(Prob<T> P, const T *__restrict__ src, double *__restrict__ dst, long long c0,
-                              long long nc)
-{
-    long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    const int G = P.G, N = P.N;
-    long long n = nc * G * N;
-    if (i >= n) return;
-    int k = (int)(i % N);
-    long long cg = i / N;
-    int g = (int)(cg % G);
-    long long c = c0 + cg / G;
-    int ix, iy, iz;
-    node_xyz(c, P.nx, P.ny, ix, iy, iz);
-    const int ki = P.mesh2int[k];  // canonical arrays are in mesh order
-    dst[i] = (double)src[((long long)ki * G + g) * P.Nc + perm_offset(P.ord[ki].d, ix, iy, iz, P.nx, P.ny, P.nz)];
+    // blockIdx.y: every gridDim.y-th chunk of ordinates
+    constexpr int KC = 32;
+    __shared__ T S[KC][65];
+    const int nbx = (P.nx + 7) / 8, nby = (P.ny + 7) / 8;
+    const int g = (int)(blockIdx.x / nbr);
+    const int b = (int)(blockIdx.x - g * nbr);
+    const int x0 = b % nbx * 8, y0 = b / nbx % nby * 8, z = z0 + b / (nbx * nby);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int N = P.N, G = P.G;
+    // canonical side: this warp's node rows r = warp + 8 i; the other: node q
+    // = tid % 64 of the run order, ordinates tid / 64 + 4 i of the chunk
+    auto node = [&](int r, long long &c) {
+        const int x = x0 + (r & 7), y = y0 + (r >> 3);
+        c = ((long long)z * P.ny + y) * P.nx + x;
+        return x < P.nx && y < P.ny && c >= c0 && c < c0 + nc;
+    };
+    for (int k0 = (int)blockIdx.y * KC; k0 < N; k0 += KC * (int)gridDim.y) {
+        auto canon_side = [&]() {
+            double v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                long long c;
+                const int r = warp + 8 * i;
+                const bool on = node(r, c) && k0 + lane < N;
+                const long long a = ((c - c0) * G + g) * N + k0 + lane;
+                if constexpr (TO_DO) v[i] = on ? canon_in[a] : 0.0;
+                else if (on) canon_out[a] = (double)S[lane][r];
+            }
+            if constexpr (TO_DO) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) S[lane][warp + 8 * i] = (T)v[i];
+            }
+        };
+        auto do_side = [&]() {
+            const int q = tid & 63;
+            T v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int kk = (tid >> 6) + 4 * i, k = k0 + kk;
+                if (k >= N) break;
+                const int ki = P.mesh2int[k], d = P.ord[ki].d;
+                const int r = d == 0 ? ((q & 7) << 3) | (q >> 3) : q;  // runs go along y in the x-class layout
+                long long c;
+                const bool on = node(r, c);
+                const long long a = ((long long)ki * G + g) * P.Nc + perm_offset(d, x0 + (r & 7), y0 + (r >> 3), z, P.nx, P.ny, P.nz);
+                if constexpr (TO_DO) {
+                    if (on) dov[a] = S[kk][r];
+                } else {
+                    v[i] = on ? dov[a] : T(0);
+                }
+            }
+            if constexpr (!TO_DO) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int kk = (tid >> 6) + 4 * i, k = k0 + kk;
+                    if (k >= N) break;
+                    const int d = P.ord[P.mesh2int[k]].d;
+                    S[kk][d == 0 ? ((q & 7) << 3) | (q >> 3) : q] = v[i];
+                }
+            }
+        };
+        if constexpr (TO_DO) canon_side();
+        else do_side();
+        __syncthreads();
+        if constexpr (TO_DO) do_side();
+        else canon_side();
+        __syncthreads();
+    }
 }
 
 template <class T>
@@ -1990,28 +2051,35 @@ cudaError_t launch_source_sums(shd_ctx *ctx, const T *Ip, T *Sp, const T *mom, c
     return cudaGetLastError();
 }
 
+template <class T, bool TO_DO>
+static cudaError_t launch_state_transpose(const shd_ctx *ctx, const double *in, double *out, T *dov, long long c0,
+                                          long long nc, cudaStream_t st)
+{
+    if (nc * ctx->G * ctx->N == 0) return cudaSuccess;
+    const long long layer = (long long)ctx->nx * ctx->ny;
+    const int z0 = (int)(c0 / layer), z1 = (int)((c0 + nc - 1) / layer);
+    const long long nbr = (long long)((ctx->nx + 7) / 8) * ((ctx->ny + 7) / 8) * (z1 - z0 + 1);
+    // few bricks: their chunks of ordinates to several CTAs (about eight an SM)
+    const int nch = (ctx->N + 31) / 32;
+    const int ny = (int)std::min<long long>(nch, std::max<long long>(1, 1216 / (nbr * ctx->G)));
+    k_state_transpose<T, TO_DO><<<dim3((unsigned)(nbr * ctx->G), (unsigned)ny), 256, 0, st>>>(make_prob<T>(ctx), in, out, dov,
+                                                                                           c0, nc, z0, nbr);
+    note_launch();
+    return cudaGetLastError();
+}
+
 template <class T>
 cudaError_t launch_canon_to_do(const shd_ctx *ctx, const double *src, T *dst, long long c0, long long nc,
                                cudaStream_t st)
 {
-    Prob<T> P = make_prob<T>(ctx);
-    long long n = nc * ctx->G * ctx->N;
-    if (n == 0) return cudaSuccess;
-    k_canon_to_do<T><<<blocks_for(n, 256), 256, 0, st>>>(P, src, dst, c0, nc);
-    note_launch();
-    return cudaGetLastError();
+    return launch_state_transpose<T, true>(ctx, src, nullptr, dst, c0, nc, st);
 }
 
 template <class T>
 cudaError_t launch_do_to_canon(const shd_ctx *ctx, const T *src, double *dst, long long c0, long long nc,
                                cudaStream_t st)
 {
-    Prob<T> P = make_prob<T>(ctx);
-    long long n = nc * ctx->G * ctx->N;
-    if (n == 0) return cudaSuccess;
-    k_do_to_canon<T><<<blocks_for(n, 256), 256, 0, st>>>(P, src, dst, c0, nc);
-    note_launch();
-    return cudaGetLastError();
+    return launch_state_transpose<T, false>(ctx, nullptr, dst, const_cast<T *>(src), c0, nc, st);
 }
 
 template <class T>
@@ -2129,14 +2197,31 @@ cudaError_t launch_ng_combine(T *x0, const T *x1, const T *x2, long long n, doub
     return cudaGetLastError();
 }
 
-template <class T>
-cudaError_t launch_rk_stage(T *I, const T *A, T *B, T *acc, long long n, double cnext, bool first, bool last,
-                            cudaStream_t st)
+template <class T, int STAGE>
+static cudaError_t launch_rk_stage_k(T *I, const T *A, T *B, T *acc, long long n, double cnext, cudaStream_t st)
 {
-    if (n == 0) return cudaSuccess;
-    k_rk_stage<T><<<blocks_for(n, 256), 256, 0, st>>>(I, A, B, acc, n, (T)cnext, first ? 1 : 0, last ? 1 : 0);
-    note_launch();
+    constexpr int V = 16 / sizeof(T);
+    const long long nv = n / V * V;
+    if (nv > 0) {
+        k_rk_stage<T, STAGE, V><<<blocks_for(nv / V, 256), 256, 0, st>>>(I, A, B, acc, 0, nv, (T)cnext);
+        note_launch();
+    }
+    if (nv < n) {
+        k_rk_stage<T, STAGE, 1><<<1, 256, 0, st>>>(I, A, B, acc, nv, n, (T)cnext);
+        note_launch();
+    }
     return cudaGetLastError();
+}
+
+template <class T>
+cudaError_t launch_rk_stage(T *I, const T *A, T *B, T *acc, long long n, double cnext, int stage, cudaStream_t st)
+{
+    switch (stage) {
+        case 0: return launch_rk_stage_k<T, 0>(I, A, B, acc, n, cnext, st);
+        case 1: return launch_rk_stage_k<T, 1>(I, A, B, acc, n, cnext, st);
+        case 2: return launch_rk_stage_k<T, 2>(I, A, B, acc, n, cnext, st);
+        default: return launch_rk_stage_k<T, 3>(I, A, B, acc, n, cnext, st);
+    }
 }
 
 #define SHD_INSTANTIATE(T)                                                                                  \
@@ -2160,8 +2245,7 @@ cudaError_t launch_rk_stage(T *I, const T *A, T *B, T *acc, long long n, double 
                                            int, double *, cudaStream_t);                                    \
     template cudaError_t launch_ng_combine<T>(T *, const T *, const T *, long long, double, double,         \
                                               cudaStream_t);                                                \
-    template cudaError_t launch_rk_stage<T>(T *, const T *, T *, T *, long long, double, bool, bool,         \
-                                            cudaStream_t);                                                  \
+    template cudaError_t launch_rk_stage<T>(T *, const T *, T *, T *, long long, double, int, cudaStream_t); \
     template cudaError_t launch_source_thermal<T>(const shd_ctx *, const T *, T *, const T *, const T *,     \
                                                   bool, int *, cudaStream_t);
 
