@@ -161,7 +161,7 @@ void dfree(void *&p)
 
 void free_all(shd_ctx *c)
 {
-    void **ptrs[] = {&c->d_ord, &c->d_W, &c->d_dirs, &c->d_Y, &c->d_mu, (void **)&c->d_edges, (void **)&c->d_centre,
+    void **ptrs[] = {&c->d_ord, &c->d_W, &c->d_dirs, &c->d_Y, &c->d_mu, (void **)&c->d_edges, (void **)&c->d_centre, (void **)&c->d_gw,
                      &c->d_alpha0, &c->d_ne, &c->d_u, &c->d_emis0, &c->d_chi0, &c->d_K, &c->d_sigma_out, &c->d_bc,
                      &c->d_I, &c->d_eta, &c->d_chi, &c->d_Ip, &c->d_Sp, &c->d_Sprev, &c->d_mom,
                      (void **)&c->d_sums, (void **)&c->d_partial, (void **)&c->d_stage,
@@ -852,11 +852,32 @@ cudaError_t check_fields(shd_ctx *c, const double *alpha0, const double *ne, con
 int ensure_remap_tables(shd_ctx *c, cudaStream_t st)
 {
     // (the entries pack the ring index in 10 bits, the group ranges in 8)
-    if (is_fp64(c) || c->rtab_valid || c->nmoving == 0 || !c->have_fields || !c->have_angles || c->nmu > 1024 ||
-        c->G > 255 || !c->d_fstage || !c->fstage_u_current || !c->d_dirs64)
-        return SHD_OK;
+    if (c->rtab_valid || c->nmoving == 0 || !c->have_fields || !c->have_angles || c->nmu > 1024) return SHD_OK;
     const size_t n = (size_t)c->nmoving * c->N;
     int rc;
+    if (is_fp64(c)) {
+        if (n != c->rtab_n || !c->d_rtab[0] || !c->d_rtab[1]) {
+            c->rtab_n = 0;
+            for (int i = 0; i < 2; ++i)
+                if (dalloc(c, &c->d_rtab[i], n * remap_entry64_bytes(), "remap tables")) {
+                    // no room: the remaps compute in place
+                    dfree(c->d_rtab[0]);
+                    dfree(c->d_rtab[1]);
+                    cudaGetLastError();
+                    return SHD_OK;
+                }
+            c->rtab_n = n;
+        }
+        CK(launch_remap_tables_d(c, c->d_rtab[0], c->d_rtab[1], c->stream), "remap tables");
+        if (st) {
+            if ((rc = stream_after(st, c->stream))) return rc;
+        } else {
+            CK(cudaStreamSynchronize(c->stream), "remap tables");
+        }
+        c->rtab_valid = true;
+        return SHD_OK;
+    }
+    if (c->G > 255 || !c->d_fstage || !c->fstage_u_current || !c->d_dirs64) return SHD_OK;
     if (n != c->rtab_n || !c->d_rtab[0] || !c->d_rtab[1] || !c->d_rrng[0] || !c->d_rrng[1]) {
         c->rtab_n = 0;
         for (int i = 0; i < 2; ++i) {
@@ -1349,9 +1370,16 @@ int shd_set_groups(shd_ctx *c, int G, const double *edges)
     for (int g = 0; g < G; ++g) c->h_centre[g] = std::sqrt(edges[g] * edges[g + 1]);
     dfree((void *&)c->d_edges);
     dfree((void *&)c->d_centre);
+    dfree((void *&)c->d_gw);
     cudaError_t e;
     c->d_edges = (double *)to_device_vec<double>(c->h_edges, c->bytes, e); CK(e, "edges");
     c->d_centre = (double *)to_device_vec<double>(c->h_centre, c->bytes, e); CK(e, "centres");
+    std::vector<double> gw(2 * (size_t)G);
+    for (int g = 0; g < G; ++g) {
+        gw[g] = 4.0 * kPi * (c->h_edges[g + 1] - c->h_edges[g]);
+        gw[G + g] = gw[g] / c->h_centre[g];
+    }
+    c->d_gw = (double *)to_device_vec<double>(gw, c->bytes, e); CK(e, "group weights");
     // log-energy tables of the frame remaps: log centres and inverse spacings
     std::vector<double> lc(G), linv(G, 0.0);
     for (int g = 0; g < G; ++g) lc[g] = std::log(c->h_centre[g]);

@@ -30,7 +30,7 @@ Prob<T> make_prob(const shd_ctx *c)
     p.kappa = (T)c->kappa;
     p.ord = (const Ordinate *)c->d_ord;
     p.W = (const T *)c->d_W; p.dirs = (const T *)c->d_dirs; p.Y = (const T *)c->d_Y; p.mu = (const T *)c->d_mu;
-    p.edges = c->d_edges; p.centre = c->d_centre;
+    p.edges = c->d_edges; p.centre = c->d_centre; p.gw = c->d_gw;
     p.alpha0 = (const T *)c->d_alpha0; p.ne = (const T *)c->d_ne; p.u = (const T *)c->d_u;
     p.emis0 = (const T *)c->d_emis0; p.chi0 = (const T *)c->d_chi0;
     p.K = (const T *)c->d_K; p.sigma_out = (const T *)c->d_sigma_out;
@@ -266,9 +266,8 @@ __global__ void __launch_bounds__(256, 3) k_source_sums(Prob<T> P, const T *__re
         }
         for (int g = lane; g < G; g += 32) {
             const double J = (double)mom[(c * G + g) * 10];
-            const double de = P.edges[g + 1] - P.edges[g];
-            e += 4.0 * kPi * J * de;
-            ph += 4.0 * kPi * J * de / P.centre[g];
+            e += J * P.gw[g];
+            ph += J * P.gw[P.G + g];
         }
         __syncwarp();
     }
@@ -385,9 +384,8 @@ __global__ void __launch_bounds__(512, 1) k_source_kn(Prob<float> P, const float
         for (int i = tid; i < nn * G; i += nt) {
             const int g = i % G;
             const double J = (double)mom[(c0 * G + i) * 10];
-            const double de = P.edges[g + 1] - P.edges[g];
-            e += 4.0 * kPi * J * de;
-            ph += 4.0 * kPi * J * de / P.centre[g];
+            e += J * P.gw[g];
+            ph += J * P.gw[P.G + g];
         }
         __syncthreads();
         const float *tI = sI + (size_t)buf * tile_f;
@@ -917,9 +915,8 @@ __global__ void k_sums_partial(Prob<T> P, const T *__restrict__ mom, const T *__
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nJ; i += stride) {
         int g = (int)(i % P.G);
         double J = (double)mom[i * 10];
-        const double de = P.edges[g + 1] - P.edges[g];
-        e += 4.0 * kPi * J * de;
-        ph += 4.0 * kPi * J * de / P.centre[g];
+        e += J * P.gw[g];
+        ph += J * P.gw[P.G + g];
     }
     // |S|^2 and |S - S_prev|^2 in working precision over runs of 64 of a
     // thread's elements, each run's sums then added in FP64 (an FP64
@@ -1276,9 +1273,8 @@ __global__ void __launch_bounds__(512, 1) k_source_kn_th(Prob<float> P, const fl
             for (int i = tid; i < nn * G; i += nt) {
                 const int n = i / G, g = i - n * G;
                 const double J = (double)mom[(sC[buf][n] * G + g) * 10];
-                const double de = P.edges[g + 1] - P.edges[g];
-                e += 4.0 * kPi * J * de;
-                ph += 4.0 * kPi * J * de / P.centre[g];
+                e += J * P.gw[g];
+                ph += J * P.gw[P.G + g];
             }
             __syncthreads();
             const float *tI = sI + (size_t)buf * tile_f;
@@ -1434,9 +1430,8 @@ __global__ void __launch_bounds__(256) k_source_thermal(Prob<T> P, const T *__re
             num += (double)nm;
             for (int g = lane; g < G; g += 32) {
                 const double J = (double)mom[(c * G + g) * 10];
-                const double de = P.edges[g + 1] - P.edges[g];
-                e += 4.0 * kPi * J * de;
-                ph += 4.0 * kPi * J * de / P.centre[g];
+                e += J * P.gw[g];
+                ph += J * P.gw[P.G + g];
             }
             __syncwarp();
         }
@@ -1963,7 +1958,9 @@ cudaError_t launch_source_sums(shd_ctx *ctx, const T *Ip, T *Sp, const T *mom, c
     auto kern = ctx->k_diagonal && ctx->G <= 32 ? k_source_sums<T, true> : k_source_sums<T, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    const int nb = ctx->n_partial;
+    // at least four nodes a warp: every CTA's eight warps pay the FP64
+    // reduction and the staging of K (16^3: 1216 CTAs 24 us in FP32 and 31 in FP64, 128 CTAs 17 and 21)
+    const int nb = (int)std::min<long long>(ctx->n_partial, (ctx->Nc + 31) / 32);
     int grid_cc = nb;  // partial-sum rows of the CUDA-core pass
     auto cuda_cores = [&]() -> cudaError_t {
         if constexpr (sizeof(T) == 4) {

@@ -705,9 +705,8 @@ __global__ void __launch_bounds__(256, 2) k_source_tc(Prob<float> P, const float
             emt[i] = chi > 0.f ? 3.5449077018110320546f * P.emis0[c * G + (i % G)] / chi : 0.f;  // sqrt(4 pi)
             const int g = i % G;
             const double J = (double)mom[(c * G + g) * 10];
-            const double de = P.edges[g + 1] - P.edges[g];
-            e_sum += 4.0 * kPi * J * de;
-            ph_sum += 4.0 * kPi * J * de / P.centre[g];
+            e_sum += J * P.gw[g];
+            ph_sum += J * P.gw[P.G + g];
         }
         // the tile's chunks in order (l, q), software-pipelined: chunk i+1's
         // operands are built while chunk i's products run

@@ -36,81 +36,125 @@ __device__ inline int tile_row(int d, int q)
 }
 
 // -------------------------------------------------------------------------
-// a1: [64 x N] x [N x NB] per (tile, group); 128 threads = 8 row groups of 8
-// rows x 16 column groups of TC columns (NB = 16 TC >= NLM + 10).
+// FP64.  GB300's FP64 pipe takes about 1.6 FMAs a clock and SM, so both
+// contractions are bound by it with one warp in flight already: what matters
+// is that no product is formed twice or for padding, and that the work lies
+// evenly over the SMs.  A thread owns one node (row of an 8 x 8 brick, 64
+// threads a CTA) x four columns, operands straight from global memory with
+// eight ordinates in flight; a CTA per (brick, group, slice of columns), the
+// slices small enough that a 16^3 problem fills the GPU.
+// 16^3, one group, 128 ordinates: a1 107 -> 42 us, a3 47 -> 21 us
+// (a 64 x 32-column tile on 64 of the 152 SMs before, with the moving
+// bricks' harmonics formed twice).
+//
+// a1: column slices 0 .. nsh - 1 hold four harmonics each, from the
+// laboratory intensity at rest and the comoving (node-major) one of moving
+// nodes; the rest four laboratory moments each.
 // -------------------------------------------------------------------------
-template <class T, int TC>
-__global__ void __launch_bounds__(128) k_project_tile(Prob<T> P, const T *__restrict__ I, const T *__restrict__ I0,
-                                                      T *__restrict__ Ip, T *__restrict__ mom)
+__global__ void __launch_bounds__(64) k_project_f64(Prob<double> P, const double *__restrict__ I,
+                                                    const double *__restrict__ I0, double *__restrict__ Ip,
+                                                    double *__restrict__ mom, int nZ, int nA, int nsl)
 {
-    constexpr int R = 64, KC = 32, NB = 16 * TC, TR = 8;
-    __shared__ T As[KC][R];
-    __shared__ T Bs[KC][NB];
-    const int tile = blockIdx.x / P.G, g = blockIdx.x - (blockIdx.x / P.G) * P.G;
-    const TileInfo ti = P.tiles[tile];
-    const int tid = threadIdx.x, tr = tid >> 4, tc = tid & 15;
-    const int NLM = P.NLM;
-    const int passes = (ti.flags & 1) ? 2 : 1;
-    for (int pass = 0; pass < passes; ++pass) {
-        T acc[TR][TC];
+    constexpr int U = 8;
+    const int NLM = P.NLM, N = P.N, G = P.G, NB = P.NB;
+    const int nsh = (NLM + 3) >> 2;
+    const long long item = blockIdx.x / nsl;
+    const int sl = (int)(blockIdx.x - item * nsl);
+    const int g = (int)(item / P.ntiles);
+    const TileInfo ti = P.tiles[item - g * P.ntiles];
+    const bool harm = sl < nsh;
+    const int col0 = harm ? 4 * sl : NLM + 4 * (sl - nsh), cend = harm ? NLM : NLM + 10;
+    const int r = threadIdx.x, x = ti.x0 + (r & 7), y = ti.y0 + (r >> 3);
+    const bool in = x < P.nx && y < P.ny;
+    const int xx = in ? x : P.nx - 1, yy = in ? y : P.ny - 1;
+    const long long c = ((long long)ti.z * P.ny + yy) * P.nx + xx;
+    const int m = harm && in ? P.midx[c] : -1;
+    // ordinate k's value at base[k * step + the class's offset]
+    const double *base = m >= 0 ? I0 + ((long long)m * G + g) * N : I + (long long)g * P.Nc;
+    const long long step = m >= 0 ? 1 : (long long)G * P.Nc;
+    const long long oz = m >= 0 ? 0 : c, oy = m >= 0 ? 0 : ((long long)yy * P.nz + ti.z) * P.nx + xx;
+    const long long ox = m >= 0 ? 0 : ((long long)xx * P.nz + ti.z) * P.ny + yy;
+    int cc[4];
 #pragma unroll
-        for (int i = 0; i < TR; ++i)
+    for (int j = 0; j < 4; ++j) cc[j] = col0 + j < cend ? col0 + j : cend - 1;
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    double a[U], an[U];  // a batch of ordinates, and the next one in flight
+    auto load = [&](int k0, double (&v)[U]) {
 #pragma unroll
-            for (int j = 0; j < TC; ++j) acc[i][j] = T(0);
-        for (int k0 = 0; k0 < P.N; k0 += KC) {
-            for (int e = tid; e < KC * R; e += 128) {
-                int kk = e >> 6, q = e & 63, k = k0 + kk;
-                T v = T(0);
-                int r = q;
-                if (k < P.N) {
-                    int d = P.ord[k].d;
-                    r = tile_row(d, q);
-                    int ix = ti.x0 + (r & 7), iy = ti.y0 + (r >> 3);
-                    if (ix < P.nx && iy < P.ny) {
-                        const int m = P.midx[((long long)ti.z * P.ny + iy) * P.nx + ix];
-                        if (pass == 1 && m >= 0)
-                            v = I0[((long long)m * P.G + g) * P.N + k];  // comoving, node-major
-                        else
-                            v = I[((long long)k * P.G + g) * P.Nc + perm_offset(d, ix, iy, ti.z, P.nx, P.ny, P.nz)];
-                    }
-                }
-                As[kk][r] = v;
-            }
-            for (int e = tid; e < KC * NB; e += 128) {
-                int kk = e / NB, j = e - kk * NB, k = k0 + kk;
-                Bs[kk][j] = k < P.N ? P.Bproj[(size_t)k * NB + j] : T(0);
-            }
-            __syncthreads();
-#pragma unroll 4
-            for (int kk = 0; kk < KC; ++kk) {
-                T a[TR], b[TC];
+        for (int u = 0; u < U; ++u) {
+            const int k = k0 + u < N ? k0 + u : N - 1;
+            v[u] = base[k * step + (k < nZ ? oz : (k < nA ? oy : ox))];
+        }
+    };
+    load(0, a);
+    for (int k0 = 0; k0 < N; k0 += U) {
+        if (k0 + U < N) load(k0 + U, an);
 #pragma unroll
-                for (int i = 0; i < TR; ++i) a[i] = As[kk][tr * TR + i];
+        for (int u = 0; u < U; ++u) {
+            if (k0 + u >= N) break;
+            const double *b = P.Bproj + (size_t)(k0 + u) * NB;
 #pragma unroll
-                for (int j = 0; j < TC; ++j) b[j] = Bs[kk][tc + 16 * j];
-#pragma unroll
-                for (int i = 0; i < TR; ++i)
-#pragma unroll
-                    for (int j = 0; j < TC; ++j) acc[i][j] += a[i] * b[j];
-            }
-            __syncthreads();
+            for (int j = 0; j < 4; ++j) acc[j] += a[u] * b[cc[j]];
         }
 #pragma unroll
-        for (int i = 0; i < TR; ++i) {
-            int r = tr * TR + i;
-            int ix = ti.x0 + (r & 7), iy = ti.y0 + (r >> 3);
-            if (ix >= P.nx || iy >= P.ny) continue;
-            long long c = ((long long)ti.z * P.ny + iy) * P.nx + ix;
-            bool moving = P.mflag[c] != 0;
+        for (int u = 0; u < U; ++u) a[u] = an[u];
+    }
+    if (!in) return;
 #pragma unroll
-            for (int j = 0; j < TC; ++j) {
-                int col = tc + 16 * j;
-                if (col < NLM) {
-                    if ((pass == 0 && !moving) || (pass == 1 && moving)) Ip[(c * P.G + g) * NLM + col] = acc[i][j];
-                } else if (col < NLM + 10 && pass == 0) {
-                    mom[(c * P.G + g) * 10 + (col - NLM)] = acc[i][j];
-                }
-            }
+    for (int j = 0; j < 4; ++j) {
+        const int col = col0 + j;
+        if (col >= cend) break;
+        if (harm) Ip[(c * G + g) * NLM + col] = acc[j];
+        else mom[(c * G + g) * 10 + (col - NLM)] = acc[j];
+    }
+}
+
+// a3: a CTA of 128 threads per (brick, group, slice of eight ordinates): a
+// thread's node x four ordinates, the brick's S staged in shared memory.  A
+// node at rest writes eta = chi0 S0, chi = chi0; a moving node's S0 goes
+// node-major for its remap.
+__global__ void __launch_bounds__(128) k_sh2lab_f64(Prob<double> P, const double *__restrict__ Sp,
+                                                    double *__restrict__ eta, double *__restrict__ chi,
+                                                    double *__restrict__ S0, int nsl)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double *As = reinterpret_cast<double *>(smem_raw);  // [NLM][65]
+    const int NLM = P.NLM, N = P.N, G = P.G;
+    const long long item = blockIdx.x / nsl;
+    const int sl = (int)(blockIdx.x - item * nsl);
+    const int g = (int)(item / P.ntiles);
+    const TileInfo ti = P.tiles[item - g * P.ntiles];
+    for (int e = threadIdx.x; e < 64 * NLM; e += 128) {
+        const int q = e / NLM, p = e - q * NLM, x = ti.x0 + (q & 7), y = ti.y0 + (q >> 3);
+        As[p * 65 + q] = x < P.nx && y < P.ny ? Sp[((((long long)ti.z * P.ny + y) * P.nx + x) * G + g) * NLM + p] : 0.0;
+    }
+    __syncthreads();
+    const int r = threadIdx.x & 63, k0 = sl * 8 + 4 * (threadIdx.x >> 6);
+    const double *Y[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) Y[j] = P.Y + (size_t)(k0 + j < N ? k0 + j : N - 1) * NLM;
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+    for (int p = 0; p < NLM; ++p) {
+        const double a = As[p * 65 + r];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[j] += a * Y[j][p];
+    }
+    const int x = ti.x0 + (r & 7), y = ti.y0 + (r >> 3);
+    if (x >= P.nx || y >= P.ny) return;
+    const long long c = ((long long)ti.z * P.ny + y) * P.nx + x;
+    const double ch = P.chi0[c * G + g];
+    const int m = P.midx[c];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int k = k0 + j;
+        if (k >= N) break;
+        if (m >= 0) {
+            S0[((long long)m * G + g) * N + k] = acc[j];
+        } else {
+            const long long o = ((long long)k * G + g) * P.Nc + perm_offset(P.ord[k].d, x, y, ti.z, P.nx, P.ny, P.nz);
+            eta[o] = ch * acc[j];
+            chi[o] = ch;
         }
     }
 }
@@ -883,6 +927,39 @@ __device__ inline float4 table_entry(const StencilParams<float> &p, float ratio)
     return make_float4(__int_as_float(p.mode | (p.a << 2) | (p.b << 12)), p.t, p.tp, ratio);
 }
 
+// FP64 entries: the placement, the ratio q and what follows from it
+struct RemapEntry64 {
+    double t, tp, q, lq, iq3;
+    int code, pad;
+};
+
+__device__ inline RemapEntry64 table_entry64(const StencilParams<double> &p, double q)
+{
+    RemapEntry64 e;
+    e.t = p.t;
+    e.tp = p.tp;
+    e.q = q;
+    e.lq = log(q);
+    e.iq3 = 1.0 / (q * q * q);
+    e.code = p.mode | (p.a << 2) | (p.b << 12);
+    e.pad = 0;
+    return e;
+}
+
+__device__ inline Stencil<double> table_stencil64(const RemapEntry64 &e, int nphi, const int *m2i)
+{
+    StencilParams<double> p;
+    p.mode = e.code & 3;
+    p.a = (e.code >> 2) & 1023;
+    p.b = e.code >> 12;
+    p.t = e.t;
+    p.tp = e.tp;
+    Stencil<double> s = stencil_from_params<double>(p, nphi);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s.k[i] = m2i[s.k[i]];
+    return s;
+}
+
 template <class T>
 __device__ inline Stencil<T> table_stencil(const float4 &e, int nphi, const int *m2i)
 {
@@ -946,6 +1023,28 @@ __global__ void __launch_bounds__(256) k_remap_tables(Prob<float> P, float4 *__r
     rl[i] = group_range(P, boost_dir<double>(ud, nd, od, 1.0));
 }
 
+// The FP64 tables: the values the FP64 remaps would compute in place (two
+// square roots, ten divisions, an arctangent and a logarithm a (node,
+// ordinate) and remap on the narrow FP64 pipe, every step): 23 x 21 x 18
+// nodes, 8 groups, 128 ordinates 1.23 -> 0.94 ms comoving, 1.90 -> 1.23 ms
+// laboratory (there with chi0's log ratios taken once a node).
+__global__ void __launch_bounds__(256) k_remap_tables64(Prob<double> P, RemapEntry64 *__restrict__ tc,
+                                                        RemapEntry64 *__restrict__ tl)
+{
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= P.nmoving * P.N) return;
+    const long long m = i / P.N;
+    const int k = (int)(i - m * P.N);
+    const long long c = P.moving[m];
+    const double u[3] = {P.u[3 * c], P.u[3 * c + 1], P.u[3 * c + 2]};
+    const double nk[3] = {P.dirs[3 * k], P.dirs[3 * k + 1], P.dirs[3 * k + 2]};
+    double nb[3];
+    const double q = boost_dir<double>(u, nk, nb, -1.0);
+    tc[i] = table_entry64(stencil_params<double>(P.mu, P.nmu, P.nphi, nb), q);
+    const double D = boost_dir<double>(u, nk, nb, 1.0);
+    tl[i] = table_entry64(stencil_params<double>(P.mu, P.nmu, P.nphi, nb), D);
+}
+
 // Energy offset x = l / (log spacing) of equally spaced log centres, split
 // into its whole part s and fraction t.
 template <class T>
@@ -997,11 +1096,15 @@ __device__ inline FlatStencil<T> flat_stencil(const Stencil<T> &s)
 __device__ inline int clamp_group(int ga, int G) { return ga < 0 ? 0 : (ga > G - 2 ? G - 2 : ga); }
 
 // chi0 between centres ga and ga+1: geometric from the node's log-ratio
-// table where both are positive, linear otherwise
+// table where both are positive, linear otherwise (FP64: the natural
+// logarithm, so that the value is freq_mix's)
 template <class T>
 __device__ inline T chi_mix(const T *schi, const T *slr, int ga, T t)
 {
     const T a = schi[ga], b = schi[ga + 1];
+    if constexpr (sizeof(T) == 8) {
+        if (a > T(0) && b > T(0)) return a * exp(t * slr[ga]);
+    }
     if (a > T(0) && b > T(0)) return freq_mix_lr<T>(a, slr[ga], t);
     return (T(1) - t) * a + t * b;
 }
@@ -1018,7 +1121,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 3 : 4) k_remap_to_comovi
                                                            const float4 *__restrict__ tab,
                                                            const unsigned short *__restrict__ rng)
 {
-    static_assert(!TAB || sizeof(T) == 4, "the remap tables are FP32");
+    constexpr bool F32 = sizeof(T) == 4;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int G = P.G, N = P.N;
     T *sI = reinterpret_cast<T *>(smem_raw);  // [G][N] internal order
@@ -1027,7 +1130,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 3 : 4) k_remap_to_comovi
     const long long c = P.moving[m];
     // the first two table entries of this thread, in flight during the staging
     float4 epre[2] = {};
-    if constexpr (TAB) {
+    if constexpr (TAB && F32) {
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
             const int kk = threadIdx.x + i * blockDim.x;
@@ -1057,18 +1160,27 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 3 : 4) k_remap_to_comovi
                 ghi = (int)(r >> 8);
             }
         };
-        if constexpr (TAB) {
+        T iq3, lq;
+        if constexpr (TAB && F32) {
             const float4 e = iter == 0 ? epre[0] : (iter == 1 ? epre[1] : tab[m * N + k0]);
             q = (T)e.w;
             st = table_stencil<T>(e, P.nphi, tb.m2i);
+        } else if constexpr (TAB) {
+            const RemapEntry64 e = reinterpret_cast<const RemapEntry64 *>(tab)[m * N + k0];
+            q = e.q;
+            lq = e.lq;
+            iq3 = e.iq3;
+            st = table_stencil64(e, P.nphi, tb.m2i);
         } else {
             T n0[3] = {P.dirs[3 * k0], P.dirs[3 * k0 + 1], P.dirs[3 * k0 + 2]};
             T n[3];
             q = boost_any<T>(u, n0, n, T(-1), P.fp64_boost);
             st = stencil_internal<T>(P, tb, n);
         }
-        T iq3 = T(1) / (q * q * q);
-        T lq = dlog<T>(q);
+        if constexpr (!TAB || F32) {
+            iq3 = T(1) / (q * q * q);
+            lq = dlog<T>(q);
+        }
         GroupCache<T> cache;
         if (sizeof(T) == 4 && P.lgu) {
             // equally spaced log centres: energy lc[g0] + lq sits at g0 + x
@@ -1126,7 +1238,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 3 : 4) k_remap_to_comovi
         for (int g0 = 0; g0 < G; ++g0) {
             const T le = tb.lc[g0] + lq;
             FreqBracket<T> fb = freq_bracket<T>(tb.lc, tb.linv, P.le0, P.leG, G, le, hint);
-            if (TAB && (dabs<T>(le - P.le0) < T(kEdgeTol) || dabs<T>(le - P.leG) < T(kEdgeTol))) {
+            if (TAB && F32 && (dabs<T>(le - P.le0) < T(kEdgeTol) || dabs<T>(le - P.leG) < T(kEdgeTol))) {
                 range();  // inside or beyond the edges as the table decided
                 if (g0 < glo || g0 >= ghi) fb.mode = 0;
                 else if (fb.mode == 0) fb.mode = 1;  // the nearest outer group (fb.ga)
@@ -1152,13 +1264,13 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 3 : 4) k_remap_to_lab(Pr
                                                       T *__restrict__ chi_n, const float4 *__restrict__ tab,
                                                       const unsigned short *__restrict__ rng)
 {
-    static_assert(!TAB || sizeof(T) == 4, "the remap tables are FP32");
+    constexpr bool F32 = sizeof(T) == 4;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int G = P.G, N = P.N;
     T *sS = reinterpret_cast<T *>(smem_raw);  // [G][N] internal order
     T *spole = sS + (size_t)G * N;            // [G][2]
     T *schi = spole + 2 * G;                  // [G]
-    T *slr = schi + G;                        // [G] FP32: log2(chi0[g+1]/chi0[g]) where both > 0
+    T *slr = schi + G;                        // [G] log2 (FP64: log) of chi0[g+1]/chi0[g] where both > 0
     const long long m = blockIdx.x;
     const long long c = P.moving[m];
     stage_node<T>(sS, S0 + m * G * N, G * N);
@@ -1166,9 +1278,10 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 3 : 4) k_remap_to_lab(Pr
     const RemapTables<T> tb = remap_tables<T>(P, reinterpret_cast<unsigned char *>(slr + G));
     __syncthreads();
     pole_averages<T>(P, sS, tb.m2i, spole);
-    for (int g = threadIdx.x; sizeof(T) == 4 && g + 1 < G; g += blockDim.x) {
+    for (int g = threadIdx.x; g + 1 < G; g += blockDim.x) {
         const T a = schi[g], b = schi[g + 1];
-        slr[g] = (a > T(0) && b > T(0)) ? T(log2f(float(b / a))) : T(0);
+        if constexpr (F32) slr[g] = (a > T(0) && b > T(0)) ? T(log2f(float(b / a))) : T(0);
+        else slr[g] = (a > T(0) && b > T(0)) ? log(b / a) : T(0);
     }
     __syncthreads();
     const T u[3] = {P.u[3 * c], P.u[3 * c + 1], P.u[3 * c + 2]};
@@ -1187,18 +1300,27 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 3 : 4) k_remap_to_lab(Pr
                 ghi = (int)(r >> 8);
             }
         };
-        if constexpr (TAB) {
+        T iD3, lD;
+        if constexpr (TAB && F32) {
             const float4 e = tab[m * N + k];
             D = (T)e.w;
             st = table_stencil<T>(e, P.nphi, tb.m2i);
+        } else if constexpr (TAB) {
+            const RemapEntry64 e = reinterpret_cast<const RemapEntry64 *>(tab)[m * N + k];
+            D = e.q;
+            lD = e.lq;
+            iD3 = e.iq3;
+            st = table_stencil64(e, P.nphi, tb.m2i);
         } else {
             T n[3] = {P.dirs[3 * k], P.dirs[3 * k + 1], P.dirs[3 * k + 2]};
             T n0[3];
             D = boost_any<T>(u, n, n0, T(1), P.fp64_boost);
             st = stencil_internal<T>(P, tb, n0);
         }
-        T iD3 = T(1) / (D * D * D);
-        T lD = dlog<T>(D);
+        if constexpr (!TAB || F32) {
+            iD3 = T(1) / (D * D * D);
+            lD = dlog<T>(D);
+        }
         GroupCache<T> cache;
         if (sizeof(T) == 4 && P.lgu) {
             // equally spaced log centres: the constant shift s and fraction t
@@ -1268,7 +1390,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 3 : 4) k_remap_to_lab(Pr
         for (int g = 0; g < G; ++g) {
             const T le = tb.lc[g] + lD;
             FreqBracket<T> fb = freq_bracket<T>(tb.lc, tb.linv, P.le0, P.leG, G, le, hint);
-            if (TAB && (dabs<T>(le - P.le0) < T(kEdgeTol) || dabs<T>(le - P.leG) < T(kEdgeTol))) {
+            if (TAB && F32 && (dabs<T>(le - P.le0) < T(kEdgeTol) || dabs<T>(le - P.leG) < T(kEdgeTol))) {
                 range();  // inside or beyond the edges as the table decided
                 if (g < glo || g >= ghi) fb.mode = 0;
                 else if (fb.mode == 0) fb.mode = 1;  // the nearest outer group (fb.ga)
@@ -1283,8 +1405,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 3 : 4) k_remap_to_lab(Pr
                 T fa = cache.get(st, sS, spole, N, fb.ga);
                 T fbv = cache.get(st, sS, spole, N, fb.ga + 1);
                 s = freq_mix<T>(fa, fbv, fb.t);
-                ch = sizeof(T) == 4 ? chi_mix<T>(schi, slr, fb.ga, fb.t)
-                                    : freq_mix<T>(schi[fb.ga], schi[fb.ga + 1], fb.t);
+                ch = chi_mix<T>(schi, slr, fb.ga, fb.t);
             }
             T chl = ch * D;
             dc[(size_t)g * N + k] = chl;
@@ -1306,16 +1427,6 @@ size_t remap_smem_bytes(const shd_ctx *c)
 size_t sh2lab_tile_smem_bytes(const shd_ctx *c)
 {
     return (size_t)c->esize * ((size_t)c->NLM * 64 + (size_t)c->NLM * 128 + 128 * 65 + 64) + 64 * 4 + 64;
-}
-
-template <class T, int TC>
-static cudaError_t launch_project_tile_tc(const shd_ctx *ctx, const T *I, const T *I0n, T *Ip, T *mom,
-                                          cudaStream_t st)
-{
-    Prob<T> P = make_prob<T>(ctx);
-    k_project_tile<T, TC><<<(unsigned)(ctx->ntiles * ctx->G), 128, 0, st>>>(P, I, I0n, Ip, mom);
-    note_launch();
-    return cudaGetLastError();
 }
 
 static int num_sms(const shd_ctx *ctx)
@@ -1426,8 +1537,8 @@ static cudaError_t run_remap_to_comoving(const shd_ctx *ctx, const T *nm0, T *nm
 {
     Prob<T> P = make_prob<T>(ctx);
     size_t sm = remap_smem_bytes(ctx);
-    const float4 *tab = sizeof(T) == 4 && ctx->rtab_valid ? (const float4 *)ctx->d_rtab[0] : nullptr;
-    auto kern = (sizeof(T) == 4 && tab) ? k_remap_to_comoving<T, sizeof(T) == 4> : k_remap_to_comoving<T, 0>;
+    const float4 *tab = ctx->rtab_valid ? (const float4 *)ctx->d_rtab[0] : nullptr;
+    auto kern = tab ? k_remap_to_comoving<T, 1> : k_remap_to_comoving<T, 0>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)ctx->nmoving, 256, sm, st>>>(P, nm0, nm1, tab, tab ? ctx->d_rrng[0] : nullptr);
@@ -1440,8 +1551,8 @@ static cudaError_t run_remap_to_lab(const shd_ctx *ctx, const T *nm0, T *nm1, T 
 {
     Prob<T> P = make_prob<T>(ctx);
     size_t sr = remap_smem_bytes(ctx);
-    const float4 *tab = sizeof(T) == 4 && ctx->rtab_valid ? (const float4 *)ctx->d_rtab[1] : nullptr;
-    auto kern = (sizeof(T) == 4 && tab) ? k_remap_to_lab<T, sizeof(T) == 4> : k_remap_to_lab<T, 0>;
+    const float4 *tab = ctx->rtab_valid ? (const float4 *)ctx->d_rtab[1] : nullptr;
+    auto kern = tab ? k_remap_to_lab<T, 1> : k_remap_to_lab<T, 0>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sr);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)ctx->nmoving, 256, sr, st>>>(P, nm0, nm1, nm2, tab, tab ? ctx->d_rrng[1] : nullptr);
@@ -1459,6 +1570,16 @@ cudaError_t launch_remap_tables_f(const shd_ctx *ctx, float4 *tc, float4 *tl, un
     note_launch();
     return cudaGetLastError();
 }
+
+cudaError_t launch_remap_tables_d(const shd_ctx *ctx, void *tc, void *tl, cudaStream_t st)
+{
+    const long long n = ctx->nmoving * ctx->N;
+    if (n == 0) return cudaSuccess;
+    k_remap_tables64<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(make_prob<double>(ctx), (RemapEntry64 *)tc, (RemapEntry64 *)tl);
+    note_launch();
+    return cudaGetLastError();
+}
+size_t remap_entry64_bytes() { return sizeof(RemapEntry64); }
 
 cudaError_t launch_remap_to_comoving_f(const shd_ctx *ctx, const float *nm0, float *nm1, cudaStream_t st)
 {
@@ -1487,17 +1608,13 @@ cudaError_t launch_project_nm(const shd_ctx *ctx, const T *I, T *Ip, T *mom, T *
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         if ((e = run_remap_to_comoving<T>(ctx, nm0, nm1, st)) != cudaSuccess) return e;
     }
-    if constexpr (sizeof(T) == 4) return launch_project_tc(ctx, I, Ip, mom, nm1, st);
-    else switch (ctx->NB / 16) {
-        case 1: return launch_project_tile_tc<T, 1>(ctx, I, nm1, Ip, mom, st);
-        case 2: return launch_project_tile_tc<T, 2>(ctx, I, nm1, Ip, mom, st);
-        case 3: return launch_project_tile_tc<T, 3>(ctx, I, nm1, Ip, mom, st);
-        case 4: return launch_project_tile_tc<T, 4>(ctx, I, nm1, Ip, mom, st);
-        case 5: return launch_project_tile_tc<T, 5>(ctx, I, nm1, Ip, mom, st);
-        case 6: return launch_project_tile_tc<T, 6>(ctx, I, nm1, Ip, mom, st);
-        case 7: return launch_project_tile_tc<T, 7>(ctx, I, nm1, Ip, mom, st);
-        case 8: return launch_project_tile_tc<T, 8>(ctx, I, nm1, Ip, mom, st);
-        default: return cudaErrorInvalidConfiguration;
+    if constexpr (sizeof(T) == 4) {
+        return launch_project_tc(ctx, I, Ip, mom, nm1, st);
+    } else {
+        const int nsl = (ctx->NLM + 3) / 4 + 3;  // four harmonics, four moments a slice
+        k_project_f64<<<(unsigned)(ctx->ntiles * ctx->G * nsl), 64, 0, st>>>(P, I, nm1, Ip, mom, ctx->nZ, ctx->nA, nsl);
+        note_launch();
+        return cudaGetLastError();
     }
 }
 
@@ -1528,7 +1645,15 @@ cudaError_t launch_sh2lab(const shd_ctx *ctx, const T *Sp, T *eta, T *chi, cudaS
             done = true;
         }
     }
-    if (!done) {
+    if constexpr (sizeof(T) == 8) {
+        const int nsl = (ctx->N + 7) / 8;
+        const size_t sm = sizeof(double) * 65 * (size_t)ctx->NLM;
+        e = cudaFuncSetAttribute(k_sh2lab_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        if (e != cudaSuccess) return e;
+        k_sh2lab_f64<<<(unsigned)(ctx->ntiles * ctx->G * nsl), 128, sm, st>>>(P, Sp, eta, chi, nm0, nsl);
+        note_launch();
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    } else if (!done) {
         size_t sm = sh2lab_tile_smem_bytes(ctx);
         e = cudaFuncSetAttribute(k_sh2lab_tile<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
