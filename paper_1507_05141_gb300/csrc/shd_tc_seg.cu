@@ -46,7 +46,7 @@ constexpr long long kSegWaitLimit = 1LL << 22;  // mbarrier polls before giving 
 constexpr int kKC = 32;                         // ordinates per chunk
 constexpr int kABatch = 8;                      // k_sh2lab_rows: A-build steps whose loads fly together
 constexpr int kBox = 128 * kKC;                 // floats per TMA box (16 KB)
-constexpr int kNConv = 256;                     // converter threads of a1
+constexpr int kNConv = 4;                       // converter warps a chunk in a1
 
 __device__ inline void split2(float a, float b, uint32_t &hi, uint32_t &lo)
 {
@@ -94,6 +94,7 @@ struct SegArgs {
     int Kp;             // slots = 32 nchunk
     int nb;             // a1: output columns (rows of Bp) of the MMA
     int accumulate;     // a1: add to I_lm / moments instead of storing
+    int nmom;           // a1: moments stored (1: J alone, all a step's sums read; 10)
     int chi_all;        // a3: chi for every row (else only boxes that hold a moving row)
     int4 chunk[16];     // {map index, first ordinate of the chunk within its class,
                         //  internal index of the class's first ordinate, ordinates in the class}
@@ -251,7 +252,13 @@ __global__ void __launch_bounds__(MAN ? 480 : 448, 1)
     if (warp < 8) {
         // ---------------- converters ----------------
         long long it = 0;
-        const int crow = (warp & 3) * 32 + lane;  // the row this thread converts in every chunk
+        // two teams of four warps take alternate chunks, so that one team's
+        // waits, fence and loads overlap the other's arithmetic; a warp
+        // converts 32 rows and arrives once (64^3 jet, with J the only moment
+        // stored: the three launches of a1 4.5 -> 3.8 ms; all eight warps on
+        // one chunk, each thread arriving for itself, before)
+        const int team = warp >> 2;
+        const int crow = (warp & 3) * 32 + lane;  // the row this thread converts
         for (long long w = blockIdx.x; w < S.nitem; w += gridDim.x) {
             // node-major destination of the row when its node moves
             float *nrow = nullptr;
@@ -265,53 +272,58 @@ __global__ void __launch_bounds__(MAN ? 480 : 448, 1)
                 }
             }
             for (int ch = 0; ch < nchunk; ++ch, ++it) {
+                if ((int)(it & 1) != team) continue;
                 const int s = (int)(it % NSTG), r = (int)(it % NR);
                 if (!wait(&sfull[s], (uint32_t)((it / NSTG) & 1))) goto conv_out;
-                if (it >= NR && !wait(&rempty[r], (uint32_t)((it / NR - 1) & 1))) goto conv_out;
                 float *Sb = stg + (size_t)s * kBox;
                 uint16_t *Ah = ring + (size_t)(2 * r) * 128 * kKC;
                 uint16_t *Al = Ah + (size_t)128 * kKC;
-                // unit = 32 rows x 8 ordinates (one core-matrix column of
-                // four core matrices): lane = row
+                // the row's 32 ordinates: four core matrices' columns
+                float v[kKC];
+                if (!ROWS) {
 #pragma unroll
-                for (int uu = 0; uu < 2; ++uu) {
-                    const int u = warp + 8 * uu;
-                    const int rq = u & 3, kb = u >> 2;
-                    const int row = rq * 32 + lane;
-                    float v[8];
-                    if (!ROWS) {
+                    for (int i = 0; i < kKC; ++i) v[i] = Sb[i * 128 + crow];
+                } else {
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) v[i] = Sb[(kb * 8 + i) * 128 + row];
-                    } else {
-                        const float4 a = *swz4(Sb, row, 2 * kb), b = *swz4(Sb, row, 2 * kb + 1);
-                        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-                        v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-                    }
-                    uint4 h, l;
-                    split2(v[0], v[1], h.x, l.x);
-                    split2(v[2], v[3], h.y, l.y);
-                    split2(v[4], v[5], h.z, l.z);
-                    split2(v[6], v[7], h.w, l.w);
-                    const int o = tc::canon_off(row, kb * 8, kKC);
-                    *reinterpret_cast<uint4 *>(&Ah[o]) = h;
-                    *reinterpret_cast<uint4 *>(&Al[o]) = l;
-                    if (!ROWS && nrow) {
-                        const int4 ci = S.chunk[ch];
-                        const int kl = ci.y + kb * 8;  // within the class
-                        float *dst = nrow + ci.z + kl;
-                        if (kl + 8 <= ci.w && ((ci.z + kl) & 3) == 0) {
-                            reinterpret_cast<float4 *>(dst)[0] = make_float4(v[0], v[1], v[2], v[3]);
-                            reinterpret_cast<float4 *>(dst)[1] = make_float4(v[4], v[5], v[6], v[7]);
-                        } else {
-#pragma unroll
-                            for (int i = 0; i < 8; ++i)
-                                if (kl + i < ci.w) dst[i] = v[i];
-                        }
+                    for (int q = 0; q < kKC / 4; ++q) {
+                        const float4 a = *swz4(Sb, crow, q);
+                        v[4 * q] = a.x; v[4 * q + 1] = a.y; v[4 * q + 2] = a.z; v[4 * q + 3] = a.w;
                     }
                 }
+                if (it >= NR && !wait(&rempty[r], (uint32_t)((it / NR - 1) & 1))) goto conv_out;
+#pragma unroll
+                for (int kb = 0; kb < kKC / 8; ++kb) {
+                    uint4 h, l;
+                    split2(v[8 * kb], v[8 * kb + 1], h.x, l.x);
+                    split2(v[8 * kb + 2], v[8 * kb + 3], h.y, l.y);
+                    split2(v[8 * kb + 4], v[8 * kb + 5], h.z, l.z);
+                    split2(v[8 * kb + 6], v[8 * kb + 7], h.w, l.w);
+                    const int o = tc::canon_off(crow, kb * 8, kKC);
+                    *reinterpret_cast<uint4 *>(&Ah[o]) = h;
+                    *reinterpret_cast<uint4 *>(&Al[o]) = l;
+                }
+                // (the stage goes back after the fence: the copy that refills it is
+                // an asynchronous-proxy write behind these reads)
                 tc::fence_proxy_async();
-                tc::mbar_arrive(&sempty[s]);
-                tc::mbar_arrive(&rfull[r]);
+                __syncwarp();
+                if (lane == 0) {
+                    tc::mbar_arrive(&sempty[s]);
+                    tc::mbar_arrive(&rfull[r]);
+                }
+                if (!ROWS && nrow) {
+                    const int4 ci = S.chunk[ch];
+                    float *dst = nrow + ci.z + ci.y;
+                    const int n = ci.w - ci.y;  // of the class left
+                    if (n >= kKC && ((ci.z + ci.y) & 3) == 0) {
+#pragma unroll
+                        for (int q = 0; q < kKC / 4; ++q)
+                            reinterpret_cast<float4 *>(dst)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < kKC; ++i)
+                            if (i < n) dst[i] = v[i];
+                    }
+                }
             }
         }
     conv_out:;
@@ -444,7 +456,7 @@ __global__ void __launch_bounds__(MAN ? 480 : 448, 1)
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
                         const int cc = col + e;
-                        o[4 * q + e] = cc < NLM ? (ip ? ip[cc] : 0.f) : (cc < NLM + 10 && mp ? mp[cc - NLM] : 0.f);
+                        o[4 * q + e] = cc < NLM ? (ip ? ip[cc] : 0.f) : (cc < NLM + S.nmom && mp ? mp[cc - NLM] : 0.f);
                     }
                 }
             };
@@ -473,7 +485,7 @@ __global__ void __launch_bounds__(MAN ? 480 : 448, 1)
                         const int cc = col + e;
                         if (cc < NLM) {
                             if (ip) put1(ip + cc, v[4 * q + e], false);
-                        } else if (cc < NLM + 10) {
+                        } else if (cc < NLM + S.nmom) {
                             if (mp) put1(mp + (cc - NLM), v[4 * q + e], false);
                         }
                     }
@@ -1229,8 +1241,8 @@ static cudaError_t run_project_seg(const shd_ctx *ctx, const Prob<float> &P, con
 
 // a1: the laboratory rows (groups A, B; moving rows also copied node-major
 // to nm0), the comoving remap nm0 -> nm1, the comoving rows of moving nodes.
-cudaError_t launch_project_seg(const shd_ctx *ctx, const float *I, float *Ip, float *mom, float *nm0, float *nm1,
-                               cudaStream_t st)
+cudaError_t launch_project_seg(const shd_ctx *ctx, const float *I, float *Ip, float *mom, int nmom, float *nm0,
+                               float *nm1, cudaStream_t st)
 {
     Prob<float> P = make_prob<float>(ctx);
     bool first = true;
@@ -1241,6 +1253,7 @@ cudaError_t launch_project_seg(const shd_ctx *ctx, const float *I, float *Ip, fl
         if (ctx->tcs_nchunk[grp] == 0 || ctx->nseg[grp] == 0) continue;
         SegArgs a = seg_args(ctx, grp);
         a.nb = ctx->NB;
+        a.nmom = nmom;
         a.accumulate = first ? 0 : 1;
         first = false;
         SegMaps maps{};

@@ -49,12 +49,13 @@ __device__ inline int tile_row(int d, int q)
 //
 // a1: column slices 0 .. nsh - 1 hold four harmonics each, from the
 // laboratory intensity at rest and the comoving (node-major) one of moving
-// nodes; the rest four laboratory moments each.  A CTA takes slice sl0 +
-// blockIdx.x mod nsl: all of them (sl0 = 0), or the three of the moments.
+// nodes; the rest four laboratory moments each (one holds J alone, nmom = 1).
+// A CTA takes slice sl0 + blockIdx.x mod nsl: all of them (sl0 = 0), or the
+// three of the moments.
 // -------------------------------------------------------------------------
 __global__ void __launch_bounds__(64) k_project_f64(Prob<double> P, const double *__restrict__ I,
                                                     const double *__restrict__ I0, double *__restrict__ Ip,
-                                                    double *__restrict__ mom, int nZ, int nA, int nsl, int sl0)
+                                                    double *__restrict__ mom, int nmom, int nZ, int nA, int nsl, int sl0)
 {
     constexpr int U = 8;
     const int NLM = P.NLM, N = P.N, G = P.G, NB = P.NB;
@@ -64,7 +65,7 @@ __global__ void __launch_bounds__(64) k_project_f64(Prob<double> P, const double
     const int g = (int)(item / P.ntiles);
     const TileInfo ti = P.tiles[item - g * P.ntiles];
     const bool harm = sl < nsh;
-    const int col0 = harm ? 4 * sl : NLM + 4 * (sl - nsh), cend = harm ? NLM : NLM + 10;
+    const int col0 = harm ? 4 * sl : NLM + 4 * (sl - nsh), cend = harm ? NLM : NLM + nmom;
     const int r = threadIdx.x, x = ti.x0 + (r & 7), y = ti.y0 + (r >> 3);
     const bool in = x < P.nx && y < P.ny;
     const int xx = in ? x : P.nx - 1, yy = in ? y : P.ny - 1;
@@ -94,6 +95,10 @@ __global__ void __launch_bounds__(64) k_project_f64(Prob<double> P, const double
         for (int u = 0; u < U; ++u) {
             if (k0 + u >= N) break;
             const double *b = P.Bproj + (size_t)(k0 + u) * NB;
+            if (cend - col0 == 1) {  // (J alone)
+                acc[0] += a[u] * b[col0];
+                continue;
+            }
 #pragma unroll
             for (int j = 0; j < 4; ++j) acc[j] += a[u] * b[cc[j]];
         }
@@ -1746,15 +1751,17 @@ cudaError_t launch_remap_to_lab_f(const shd_ctx *ctx, const float *nm0, float *n
 }
 
 // Moving nodes first: brick transpose of I into nm0, comoving remap into
-// nm1; then the projection contraction (reading nm1 for moving rows).
+// nm1; then the projection contraction (reading nm1 for moving rows).  The
+// caller needs nmom moments: 10, or 1 (J, all that a step's sums read; kernels
+// that compute the others beside it may store them).
 template <class T>
-cudaError_t launch_project_nm(const shd_ctx *ctx, const T *I, T *Ip, T *mom, T *nm0, T *nm1, cudaStream_t st)
+cudaError_t launch_project_nm(const shd_ctx *ctx, const T *I, T *Ip, T *mom, int nmom, T *nm0, T *nm1, cudaStream_t st)
 {
     Prob<T> P = make_prob<T>(ctx);
     cudaError_t e;
     if constexpr (sizeof(T) == 4) {
         // the segment kernels write the moving rows node-major themselves
-        if (seg_usable(ctx)) return launch_project_seg(ctx, I, Ip, mom, nm0, nm1, st);
+        if (seg_usable(ctx)) return launch_project_seg(ctx, I, Ip, mom, nmom, nm0, nm1, st);
         if (!tc_usable(ctx)) return launch_project_f32(ctx, I, Ip, mom, nm0, nm1, st);
     }
     if (ctx->nmoving > 0) {
@@ -1766,17 +1773,18 @@ cudaError_t launch_project_nm(const shd_ctx *ctx, const T *I, T *Ip, T *mom, T *
     if constexpr (sizeof(T) == 4) {
         return launch_project_tc(ctx, I, Ip, mom, nm1, st);
     } else {
-        const int nsl = (ctx->NLM + 3) / 4 + 3;  // four harmonics, four moments a slice
-        k_project_f64<<<(unsigned)(ctx->ntiles * ctx->G * nsl), 64, 0, st>>>(P, I, nm1, Ip, mom, ctx->nZ, ctx->nA, nsl, 0);
+        const int nsl = (ctx->NLM + 3) / 4 + (nmom + 3) / 4;  // four harmonics, four moments a slice
+        k_project_f64<<<(unsigned)(ctx->ntiles * ctx->G * nsl), 64, 0, st>>>(P, I, nm1, Ip, mom, nmom, ctx->nZ,
+                                                                              ctx->nA, nsl, 0);
         note_launch();
         return cudaGetLastError();
     }
 }
 
 template <class T>
-cudaError_t launch_project(const shd_ctx *ctx, const T *I, T *Ip, T *mom, cudaStream_t st)
+cudaError_t launch_project(const shd_ctx *ctx, const T *I, T *Ip, T *mom, int nmom, cudaStream_t st)
 {
-    return launch_project_nm<T>(ctx, I, Ip, mom, (T *)ctx->d_nm[0], (T *)ctx->d_nm[1], st);
+    return launch_project_nm<T>(ctx, I, Ip, mom, nmom, (T *)ctx->d_nm[0], (T *)ctx->d_nm[1], st);
 }
 
 template <bool PAIR, class TO>
@@ -1801,7 +1809,7 @@ template <class T, class TO>
 cudaError_t launch_moments(const shd_ctx *ctx, const T *I, TO *mom, cudaStream_t st)
 {
     if constexpr (sizeof(T) == 8) {
-        k_project_f64<<<(unsigned)(ctx->ntiles * ctx->G * 3), 64, 0, st>>>(make_prob<double>(ctx), I, nullptr, nullptr, mom,
+        k_project_f64<<<(unsigned)(ctx->ntiles * ctx->G * 3), 64, 0, st>>>(make_prob<double>(ctx), I, nullptr, nullptr, mom, 10,
                                                                             ctx->nZ, ctx->nA, 3, (ctx->NLM + 3) / 4);
         note_launch();
         return cudaGetLastError();
@@ -1865,7 +1873,7 @@ template <class T>
 cudaError_t launch_project_scratch(const shd_ctx *ctx, const T *I, T *Ip, T *mom, T *scratch, cudaStream_t st)
 {
     T *nm0 = scratch, *nm1 = scratch + (size_t)ctx->nmoving * ctx->G * ctx->N;
-    return launch_project_nm<T>(ctx, I, Ip, mom, nm0, nm1, st);
+    return launch_project_nm<T>(ctx, I, Ip, mom, 10, nm0, nm1, st);
 }
 
 template cudaError_t launch_project_scratch<double>(const shd_ctx *, const double *, double *, double *, double *,
@@ -1876,8 +1884,8 @@ template cudaError_t launch_project_scratch<float>(const shd_ctx *, const float 
 template cudaError_t launch_moments<double, double>(const shd_ctx *, const double *, double *, cudaStream_t);
 template cudaError_t launch_moments<float, double>(const shd_ctx *, const float *, double *, cudaStream_t);
 template cudaError_t launch_moments<float, float>(const shd_ctx *, const float *, float *, cudaStream_t);
-template cudaError_t launch_project<double>(const shd_ctx *, const double *, double *, double *, cudaStream_t);
-template cudaError_t launch_project<float>(const shd_ctx *, const float *, float *, float *, cudaStream_t);
+template cudaError_t launch_project<double>(const shd_ctx *, const double *, double *, double *, int, cudaStream_t);
+template cudaError_t launch_project<float>(const shd_ctx *, const float *, float *, float *, int, cudaStream_t);
 template cudaError_t launch_sh2lab<double>(const shd_ctx *, const double *, double *, double *, cudaStream_t, bool);
 template cudaError_t launch_sh2lab<float>(const shd_ctx *, const float *, float *, float *, cudaStream_t, bool);
 
