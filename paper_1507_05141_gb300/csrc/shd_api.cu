@@ -382,7 +382,16 @@ int upload_seg_operands(shd_ctx *c, const std::vector<double> &Bp)
         const int bw = pow2_box(na), bh = 128 / bw;
         c->seg_bw[grp] = bw;
         std::vector<int> seg;
-        for (int pl = 0; pl < nplane; ++pl)
+        // no tensor map strides the planes: runs of 128 nodes of each, no box
+        const int run = seg_manual(c) ? na * nbb : 0;
+        for (int pl = 0; pl < nplane && run; ++pl)
+            for (int i0 = 0; i0 < run; i0 += 128) {
+                seg.push_back(pl);
+                seg.push_back(i0);
+                seg.push_back(0);
+                seg.push_back(0);
+            }
+        for (int pl = 0; pl < nplane && !run; ++pl)
             for (int b0 = 0; b0 < nbb; b0 += bh)
                 for (int a0 = 0; a0 < na; a0 += bw) {
                     seg.push_back(pl);

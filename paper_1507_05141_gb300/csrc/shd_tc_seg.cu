@@ -85,11 +85,11 @@ struct SegMaps {
 
 // What one launch of the segment / rows kernels covers.
 struct SegArgs {
-    const int4 *segs;   // segment mode: {plane, a0, b0, 0} (a fastest in the box)
+    const int4 *segs;   // segment mode: {plane, a0, b0, 0} (a fastest in the box); runs: {plane, first node, 0, 0}
     long long nitem;    // segment mode: segments x G; rows mode: ceil(rows / 128)
     long long nrows;    // rows mode: nmoving x G
     int groupB;         // segment mode: 0 = group A (plane z, a = x, b = y); 1 = B (plane x, a = y, b = z)
-    int bw;             // segment mode: box width along a (a power of two, 4..128)
+    int bw;             // segment mode: box width along a (a power of two, 4..128); 0: runs of the plane's nodes
     int nchunk;         // chunks of 32 slots
     int Kp;             // slots = 32 nchunk
     int nb;             // a1: output columns (rows of Bp) of the MMA
@@ -100,12 +100,32 @@ struct SegArgs {
                         //  internal index of the class's first ordinate, ordinates in the class}
 };
 
+// Row r of a tile as (a, b) of its plane: a box, or a run of 128 nodes in
+// plane order (b past the plane where the last run ends).  Runs are for the
+// planes whose rows no tensor map can stride, where every row is addressed by
+// itself anyway: they waste nothing but the last run's end, where 64 x 2 boxes
+// leave half of a 33 x 33 plane's tile rows empty.  a1 and a3, boxes -> runs:
+// 33^3, 32 groups 2.76 -> 2.18 and 3.55 -> 2.92 ms; 45^3, 12 groups 1.34 ->
+// 1.15 and 1.76 -> 1.51; 50^3, 16 groups 3.45 -> 3.33 and 4.38 -> 4.00.
+__device__ inline void seg_ab(const Prob<float> &P, const SegArgs &S, int4 sd, int r, int &a, int &b)
+{
+    if (S.bw) {
+        a = sd.y + (r & (S.bw - 1));
+        b = sd.z + r / S.bw;
+    } else {
+        const int n = S.groupB ? P.ny : P.nx, i = sd.y + r;
+        b = i / n;
+        a = i - b * n;
+    }
+}
+
 // Index of row r's node within the sweep layout of the class behind map
 // `mi` of the tile's group (group A: 0 = z-class (x, y, z), 1 = y-class
 // (x, z, y); group B: the x-class (y, z, x)); -1 outside the grid.
 __device__ inline long long seg_li(const Prob<float> &P, const SegArgs &S, int4 sd, int r, int mi)
 {
-    const int a = sd.y + (r & (S.bw - 1)), b = sd.z + r / S.bw;
+    int a, b;
+    seg_ab(P, S, sd, r, a, b);
     if (!S.groupB) {
         if (a >= P.nx || b >= P.ny) return -1;
         return mi == 0 ? ((long long)sd.x * P.ny + b) * P.nx + a : ((long long)b * P.nz + sd.x) * P.nx + a;
@@ -131,7 +151,8 @@ __device__ inline void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n"
 // Node of row r of a segment tile; false outside the grid.
 __device__ inline bool seg_node(const Prob<float> &P, const SegArgs &S, int4 sd, int r, long long &c)
 {
-    const int a = sd.y + (r & (S.bw - 1)), b = sd.z + r / S.bw;
+    int a, b;
+    seg_ab(P, S, sd, r, a, b);
     int x, y, z;
     if (!S.groupB) {
         x = a; y = b; z = sd.x;
@@ -899,7 +920,7 @@ __global__ void __launch_bounds__(672, 1) k_sh2lab_ws(Prob<float> P, const __gri
             const int pb = (int)(it & 1);
             const int4 sd = S.segs[sg];
             const int r0 = quad * 32;
-            const int as = sd.y + r0 % S.bw, bs = sd.z + r0 / S.bw;
+            const int as = MAN ? 0 : sd.y + r0 % S.bw, bs = MAN ? 0 : sd.z + r0 / S.bw;
             if (!wait(&metaFull[pb], (uint32_t)((it >> 1) & 1))) break;
             const float chr = mchi[pb * 128 + r];
             const int m = mrow[pb * 128 + r];
@@ -1175,7 +1196,7 @@ static SegArgs seg_args(const shd_ctx *c, int grp)
     a.segs = (const int4 *)c->d_seg[grp];
     a.nitem = c->nseg[grp] * c->G;
     a.groupB = grp;
-    a.bw = c->seg_bw[grp];
+    a.bw = seg_manual(c) ? 0 : c->seg_bw[grp];
     a.nchunk = c->tcs_nchunk[grp];
     a.Kp = c->tcs_Kp[grp];
     for (int i = 0; i < a.nchunk; ++i) {
