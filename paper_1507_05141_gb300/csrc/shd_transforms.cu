@@ -95,10 +95,6 @@ __global__ void __launch_bounds__(64) k_project_f64(Prob<double> P, const double
         for (int u = 0; u < U; ++u) {
             if (k0 + u >= N) break;
             const double *b = P.Bproj + (size_t)(k0 + u) * NB;
-            if (cend - col0 == 1) {  // (J alone)
-                acc[0] += a[u] * b[col0];
-                continue;
-            }
 #pragma unroll
             for (int j = 0; j < 4; ++j) acc[j] += a[u] * b[cc[j]];
         }
