@@ -397,7 +397,7 @@ def bench_ours(args):
             "sweep_schedule": sweep_sched,
             "plain_fp32": plain,
             "err_vs_fp64_oracle": errors,
-            "roofline": {"kernel": "k_sweep_pp", "bound": "hbm", "achieved": achieved, "peak": peak,
+            "roofline": {"kernel": "k_sweep_col", "bound": "hbm", "achieved": achieved, "peak": peak,
                          "unit": "GB/s", "frac": achieved / peak, "traffic": traffic,
                          "traffic_ratio": (traffic / sweep_bytes) if traffic else None,
                          "peak_kind": peak_kind,
