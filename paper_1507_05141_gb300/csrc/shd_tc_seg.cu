@@ -206,6 +206,7 @@ __global__ void __launch_bounds__(MAN ? 480 : 448, 1)
                   const uint16_t *__restrict__ gBh, const uint16_t *__restrict__ gBl, int *err)
 {
     static_assert(!(MAN && ROWS), "rows mode always has a tensor map");
+    static_assert(NR % 2 == 0, "a ring slot is one converter team's");
     constexpr uint32_t ACC_COLS = 128;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     if (tc::smem_u32(smem_raw) & 1023) {  // the swizzled staging needs 1024-byte alignment
@@ -240,7 +241,7 @@ __global__ void __launch_bounds__(MAN ? 480 : 448, 1)
     if (tid == 0) {
         for (int i = 0; i < NSTG; ++i) {
             tc::mbar_init(&sfull[i], MAN ? 64 : 1);
-            tc::mbar_init(&sempty[i], kNConv);
+            tc::mbar_init(&sempty[i], NSTG & 1 ? 2 * kNConv : kNConv);
         }
         for (int i = 0; i < NR; ++i) {
             tc::mbar_init(&rfull[i], kNConv);
@@ -277,7 +278,13 @@ __global__ void __launch_bounds__(MAN ? 480 : 448, 1)
         // waits, fence and loads overlap the other's arithmetic; a warp
         // converts 32 rows and arrives once (64^3 jet, with J the only moment
         // stored: the three launches of a1 4.5 -> 3.8 ms; all eight warps on
-        // one chunk, each thread arriving for itself, before)
+        // one chunk, each thread arriving for itself, before).  A wait tells two
+        // consecutive phases of a barrier apart, no more, so a team must not miss
+        // one: with an even NSTG a stage is always the same team's, with an odd
+        // one a team also waits for the chunks it skips and hands their stage
+        // back, which keeps the copy after next from landing in between (36 x 40
+        // x 40, 16 groups, 448 slots: a1 2.43 ms with three stages so, 2.65 with
+        // two, 2.50 before the teams).  NR is even.
         const int team = warp >> 2;
         const int crow = (warp & 3) * 32 + lane;  // the row this thread converts
         for (long long w = blockIdx.x; w < S.nitem; w += gridDim.x) {
@@ -293,8 +300,14 @@ __global__ void __launch_bounds__(MAN ? 480 : 448, 1)
                 }
             }
             for (int ch = 0; ch < nchunk; ++ch, ++it) {
-                if ((int)(it & 1) != team) continue;
                 const int s = (int)(it % NSTG), r = (int)(it % NR);
+                if ((int)(it & 1) != team) {
+                    if constexpr (NSTG & 1) {
+                        if (!wait(&sfull[s], (uint32_t)((it / NSTG) & 1))) goto conv_out;
+                        if (lane == 0) tc::mbar_arrive(&sempty[s]);
+                    }
+                    continue;
+                }
                 if (!wait(&sfull[s], (uint32_t)((it / NSTG) & 1))) goto conv_out;
                 float *Sb = stg + (size_t)s * kBox;
                 uint16_t *Ah = ring + (size_t)(2 * r) * 128 * kKC;
@@ -1076,10 +1089,12 @@ static size_t sh2lab_ws_smem(int Kp, int Kq)
     return (size_t)4 * Kp * Kq + (size_t)4 * 128 * Kq + (size_t)16 * 1024 * 4 + 2 * 128 * (4 + 4) + 10 * 8 + 8;
 }
 
-// staging / ring depths that fit: 0 when nothing does
+// staging / ring depths that fit: 0 when nothing does (a third ring slot where
+// two fit gives nothing: 40^3, 16 groups, L = 6, rows of 416 ordinates 2.18 ms
+// with either)
 static int pick_depths(int nb, int Kp, int &nstg, int &nr)
 {
-    const int opts[4][2] = {{4, 4}, {4, 3}, {4, 2}, {3, 2}};
+    const int opts[3][2] = {{4, 4}, {4, 2}, {3, 2}};
     for (auto &o : opts)
         if (project_seg_smem(nb, Kp, o[0], o[1]) <= kSegSmemLimit) {
             nstg = o[0];
@@ -1248,8 +1263,7 @@ static cudaError_t run_project_seg(const shd_ctx *ctx, const Prob<float> &P, con
     if (!pick_depths(a.nb, a.Kp, nstg, nr)) return cudaErrorInvalidConfiguration;
     const size_t sm = project_seg_smem(a.nb, a.Kp, nstg, nr);
     auto kern = nr == 4 ? k_project_seg<4, 4, ROWS, MAN>
-                        : (nr == 3 ? k_project_seg<4, 3, ROWS, MAN>
-                                   : (nstg == 4 ? k_project_seg<4, 2, ROWS, MAN> : k_project_seg<3, 2, ROWS, MAN>));
+                        : (nstg == 4 ? k_project_seg<4, 2, ROWS, MAN> : k_project_seg<3, 2, ROWS, MAN>);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     int grid = num_sms_seg(ctx);
