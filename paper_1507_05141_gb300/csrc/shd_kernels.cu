@@ -809,7 +809,7 @@ __global__ void __launch_bounds__(1024, 1) k_sweep_bez(Prob<T> P, T *__restrict_
             if (j >= plane) break;
             const T ct = Ch[u] + kap;
             Pair2<T> v;
-            v.x = ct > T(0) ? (Et[u] + kap * In[u]) * recip<T>(ct) : T(0);
+            v.x = ct > T(0) ? quot<T>(Et[u] + kap * In[u], ct) : T(0);
             v.y = ct;
             dst[j] = v;
         }
@@ -863,7 +863,7 @@ __global__ void __launch_bounds__(1024, 1) k_sweep_bez(Prob<T> P, T *__restrict_
                 if (p == 0 || ((fin >> u) & 1u)) {
                     inew = bc_full ? P.bc[pb + j] : bc_iso;
                     // the downwind slope; no derivative (NaN) without a downwind point
-                    dP = has_d ? (xd > T(0) ? (sD - sP) * recip<T>(xd) : T(0)) : T(NAN);
+                    dP = has_d ? (xd > T(0) ? bounded_slope<T>(quot<T>(sD - sP, xd)) : T(0)) : T(NAN);
                 } else {
                     const Quad4<T> q00 = up[j], q10 = up[j - d1], q01 = up[j - d2], q11 = up[j - d1 - d2];
                     const T iu = w00 * q00.x + w10 * q10.x + w01 * q01.x + w11 * q11.x;
@@ -876,17 +876,17 @@ __global__ void __launch_bounds__(1024, 1) k_sweep_bez(Prob<T> P, T *__restrict_
                     if (!isnan(q01.w)) { dsum += w01 * q01.w; dw += w01; }
                     if (!isnan(q11.w)) { dsum += w11 * q11.w; dw += w11; }
                     const T x = s * T(0.5) * (cu + cP);
-                    const T rx = recip<T>(x);
-                    const T slope = x > T(0) ? (sP - su) * rx : T(0);
-                    const T du = dw > T(0) ? dsum * recip<T>(dw) : slope;
+                    const T slope = x > T(0) ? bounded_slope<T>(quot<T>(sP - su, x)) : T(0);
+                    const T du = dw > T(0) ? quot<T>(dsum, dw) : slope;
                     dP = slope;
                     if (has_d)
-                        dP = (x > T(0) && xd > T(0)) ? fb_derivative<T>(slope, (sD - sP) * recip<T>(xd), x, xd) : T(0);
-                    const T x3 = x * T(1.0 / 3.0);
-                    const T Cu = clamp_between<T>(su + x3 * du, su, sP);
-                    const T Cp = clamp_between<T>(sP - x3 * dP, su, sP);
+                        dP = (x > T(0) && xd > T(0))
+                                 ? fb_derivative<T>(slope, bounded_slope<T>(quot<T>(sD - sP, xd)), x, xd)
+                                 : T(0);
+                    const T Cu = clamp_between<T>(su + x * du * T(1.0 / 3.0), su, sP);
+                    const T Cp = clamp_between<T>(sP - x * dP * T(1.0 / 3.0), su, sP);
                     T e, wU, wCU, wCP, wP;
-                    bezier_weights<T>(x, rx, e, wU, wCU, wCP, wP);
+                    bezier_weights<T>(x, e, wU, wCU, wCP, wP);
                     inew = iu * e + wU * su + wCU * Cu + wCP * Cp + wP * sP;
                 }
                 Quad4<T> v;
