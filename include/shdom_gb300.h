@@ -234,17 +234,16 @@ int shd_solve_static(shd_ctx *ctx, double rel_tol, int max_iter, int *iters_out,
 /* Laboratory moments of the current state:
  *   J [c][g], H [c][g][3], K [c][g][6] (xx, yy, zz, xy, xz, yz) -- all
  * divided by 4 pi so that J is the mean intensity -- and the comoving SH
- * projection Ish [c][g][p].  Any output may be NULL.  Stage a1 is run only
- * for Ish, and gives the moments with it; without Ish they are plain sums over
- * the ordinates, in SHD_MIXED some 1e-6 closer to the exact ones than a1's.
- * Synchronous. */
+ * projection Ish [c][g][p].  Any output may be NULL.  The moments are plain
+ * sums over the ordinates, the same whichever outputs are asked for; stage a1
+ * is run only for Ish.  Synchronous. */
 int shd_get_moments(shd_ctx *ctx, double *J, double *H, double *K, double *Ish);
 
 /* The same moments of the current state (Sec. 2) into caller-owned device
  * memory: dev_mom [c][g][10] doubles on ctx's device, J, H_x, H_y, H_z, K_xx,
  * K_yy, K_zz, K_xy, K_xz, K_yz per node and group, divided by 4 pi, the values
- * shd_get_moments returns without Ish (single-precision results widened
- * exactly).  Asynchronous on cuda_stream (NULL = the context's stream),
+ * shd_get_moments returns (single-precision results widened exactly).
+ * Asynchronous on cuda_stream (NULL = the context's stream),
  * ordered after the context's earlier work and before its later work; nothing
  * is copied to the host.  Errors: SHD_ERR_ARG (dev_mom NULL), SHD_ERR_STATE
  * (not configured, no state). */

@@ -947,7 +947,7 @@ int step_once(shd_ctx *c, cudaStream_t st, cudaEvent_t *ev, const std::function<
 {
     const bool tm = ev != nullptr;
     if (tm) CK(cudaEventRecord(ev[0], st), "event");
-    CK(launch_project<T>(c, (const T *)c->d_I, (T *)c->d_Ip, (T *)c->d_mom, 1, st), "project");
+    CK(launch_project<T>(c, (const T *)c->d_I, (T *)c->d_Ip, (T *)c->d_mom, st), "project");
     if (tm) CK(cudaEventRecord(ev[1], st), "event");
     if (source_sums_usable<T>(c)) {
         // a2 with the a5 partials in the same pass; the sums stage is the final reduction
@@ -1890,15 +1890,16 @@ int shd_get_moments(shd_ctx *c, double *J, double *H, double *K, double *Ish)
     if (!c->have_state) return fail(SHD_ERR_STATE, "state not set");
     size_t nCG = (size_t)c->Nc * c->G;
     std::vector<double> mom(nCG * 10);
-    // a1 only for I_lm, its moments with it; else the kernel of shd_get_moments_dev
+    // the moments by their own kernel whether or not I_lm is asked for, so that
+    // a caller gets the same values from every call; a1 only for I_lm
     if (is_fp64(c)) {
-        if (Ish) CK(launch_project<double>(c, (const double *)c->d_I, (double *)c->d_Ip, (double *)c->d_mom, 10, c->stream), "project");
-        else CK((launch_moments<double, double>(c, (const double *)c->d_I, (double *)c->d_mom, c->stream)), "moments");
+        if (Ish) CK(launch_project<double>(c, (const double *)c->d_I, (double *)c->d_Ip, (double *)c->d_mom, c->stream), "project");
+        CK((launch_moments<double, double>(c, (const double *)c->d_I, (double *)c->d_mom, c->stream)), "moments");
         if ((rc = download_reals<double>(c, c->d_mom, mom.data(), nCG * 10))) return rc;
         if (Ish && (rc = download_reals<double>(c, c->d_Ip, Ish, nCG * c->NLM))) return rc;
     } else {
-        if (Ish) CK(launch_project<float>(c, (const float *)c->d_I, (float *)c->d_Ip, (float *)c->d_mom, 10, c->stream), "project");
-        else CK((launch_moments<float, float>(c, (const float *)c->d_I, (float *)c->d_mom, c->stream)), "moments");
+        if (Ish) CK(launch_project<float>(c, (const float *)c->d_I, (float *)c->d_Ip, (float *)c->d_mom, c->stream), "project");
+        CK((launch_moments<float, float>(c, (const float *)c->d_I, (float *)c->d_mom, c->stream)), "moments");
         if ((rc = download_reals<float>(c, c->d_mom, mom.data(), nCG * 10))) return rc;
         if (Ish && (rc = download_reals<float>(c, c->d_Ip, Ish, nCG * c->NLM))) return rc;
     }

@@ -83,6 +83,10 @@ static int project_noalloc(shd_ctx *c, void *dev_Ish, void *dev_mom, void *cuda_
     else
         e = launch_project_scratch<float>(c, (const float *)c->d_I, (float *)dev_Ish, (float *)dev_mom,
                                           (float *)scratch, st);
+    // the moments as shd_get_moments takes them (no scratch)
+    if (e == cudaSuccess)
+        e = c->precision == SHD_FP64 ? launch_moments<double, double>(c, (const double *)c->d_I, (double *)dev_mom, st)
+                                     : launch_moments<float, float>(c, (const float *)c->d_I, (float *)dev_mom, st);
     if (e != cudaSuccess) {
         snprintf(g_msg, sizeof(g_msg), "launch: %s", cudaGetErrorString(e));
         return SHD_ERR_CUDA;

@@ -94,7 +94,6 @@ struct SegArgs {
     int Kp;             // slots = 32 nchunk
     int nb;             // a1: output columns (rows of Bp) of the MMA
     int accumulate;     // a1: add to I_lm / moments instead of storing
-    int nmom;           // a1: moments stored (1: J alone, all a step's sums read; 10)
     int chi_all;        // a3: chi for every row (else only boxes that hold a moving row)
     int4 chunk[16];     // {map index, first ordinate of the chunk within its class,
                         //  internal index of the class's first ordinate, ordinates in the class}
@@ -490,7 +489,7 @@ __global__ void __launch_bounds__(MAN ? 480 : 448, 1)
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
                         const int cc = col + e;
-                        o[4 * q + e] = cc < NLM ? (ip ? ip[cc] : 0.f) : (cc < NLM + S.nmom && mp ? mp[cc - NLM] : 0.f);
+                        o[4 * q + e] = cc < NLM ? (ip ? ip[cc] : 0.f) : (cc == NLM && mp ? mp[cc - NLM] : 0.f);
                     }
                 }
             };
@@ -519,7 +518,7 @@ __global__ void __launch_bounds__(MAN ? 480 : 448, 1)
                         const int cc = col + e;
                         if (cc < NLM) {
                             if (ip) put1(ip + cc, v[4 * q + e], false);
-                        } else if (cc < NLM + S.nmom) {
+                        } else if (cc == NLM) {
                             if (mp) put1(mp + (cc - NLM), v[4 * q + e], false);
                         }
                     }
@@ -1276,8 +1275,8 @@ static cudaError_t run_project_seg(const shd_ctx *ctx, const Prob<float> &P, con
 
 // a1: the laboratory rows (groups A, B; moving rows also copied node-major
 // to nm0), the comoving remap nm0 -> nm1, the comoving rows of moving nodes.
-cudaError_t launch_project_seg(const shd_ctx *ctx, const float *I, float *Ip, float *mom, int nmom, float *nm0,
-                               float *nm1, cudaStream_t st)
+cudaError_t launch_project_seg(const shd_ctx *ctx, const float *I, float *Ip, float *mom, float *nm0, float *nm1,
+                               cudaStream_t st)
 {
     Prob<float> P = make_prob<float>(ctx);
     bool first = true;
@@ -1288,7 +1287,6 @@ cudaError_t launch_project_seg(const shd_ctx *ctx, const float *I, float *Ip, fl
         if (ctx->tcs_nchunk[grp] == 0 || ctx->nseg[grp] == 0) continue;
         SegArgs a = seg_args(ctx, grp);
         a.nb = ctx->NB;
-        a.nmom = nmom;
         a.accumulate = first ? 0 : 1;
         first = false;
         SegMaps maps{};

@@ -1747,17 +1747,17 @@ cudaError_t launch_remap_to_lab_f(const shd_ctx *ctx, const float *nm0, float *n
 }
 
 // Moving nodes first: brick transpose of I into nm0, comoving remap into
-// nm1; then the projection contraction (reading nm1 for moving rows).  The
-// caller needs nmom moments: 10, or 1 (J, all that a step's sums read; kernels
-// that compute the others beside it may store them).
+// nm1; then the projection contraction (reading nm1 for moving rows).  Of the
+// moments J is stored, all that a step's sums read (kernels that compute the
+// others beside it may store them); launch_moments gives all ten.
 template <class T>
-cudaError_t launch_project_nm(const shd_ctx *ctx, const T *I, T *Ip, T *mom, int nmom, T *nm0, T *nm1, cudaStream_t st)
+cudaError_t launch_project_nm(const shd_ctx *ctx, const T *I, T *Ip, T *mom, T *nm0, T *nm1, cudaStream_t st)
 {
     Prob<T> P = make_prob<T>(ctx);
     cudaError_t e;
     if constexpr (sizeof(T) == 4) {
         // the segment kernels write the moving rows node-major themselves
-        if (seg_usable(ctx)) return launch_project_seg(ctx, I, Ip, mom, nmom, nm0, nm1, st);
+        if (seg_usable(ctx)) return launch_project_seg(ctx, I, Ip, mom, nm0, nm1, st);
         if (!tc_usable(ctx)) return launch_project_f32(ctx, I, Ip, mom, nm0, nm1, st);
     }
     if (ctx->nmoving > 0) {
@@ -1769,8 +1769,8 @@ cudaError_t launch_project_nm(const shd_ctx *ctx, const T *I, T *Ip, T *mom, int
     if constexpr (sizeof(T) == 4) {
         return launch_project_tc(ctx, I, Ip, mom, nm1, st);
     } else {
-        const int nsl = (ctx->NLM + 3) / 4 + (nmom + 3) / 4;  // four harmonics, four moments a slice
-        k_project_f64<<<(unsigned)(ctx->ntiles * ctx->G * nsl), 64, 0, st>>>(P, I, nm1, Ip, mom, nmom, ctx->nZ,
+        const int nsl = (ctx->NLM + 3) / 4 + 1;  // four harmonics a slice, and J's
+        k_project_f64<<<(unsigned)(ctx->ntiles * ctx->G * nsl), 64, 0, st>>>(P, I, nm1, Ip, mom, 1, ctx->nZ,
                                                                               ctx->nA, nsl, 0);
         note_launch();
         return cudaGetLastError();
@@ -1778,9 +1778,9 @@ cudaError_t launch_project_nm(const shd_ctx *ctx, const T *I, T *Ip, T *mom, int
 }
 
 template <class T>
-cudaError_t launch_project(const shd_ctx *ctx, const T *I, T *Ip, T *mom, int nmom, cudaStream_t st)
+cudaError_t launch_project(const shd_ctx *ctx, const T *I, T *Ip, T *mom, cudaStream_t st)
 {
-    return launch_project_nm<T>(ctx, I, Ip, mom, nmom, (T *)ctx->d_nm[0], (T *)ctx->d_nm[1], st);
+    return launch_project_nm<T>(ctx, I, Ip, mom, (T *)ctx->d_nm[0], (T *)ctx->d_nm[1], st);
 }
 
 template <bool PAIR, class TO>
@@ -1869,7 +1869,7 @@ template <class T>
 cudaError_t launch_project_scratch(const shd_ctx *ctx, const T *I, T *Ip, T *mom, T *scratch, cudaStream_t st)
 {
     T *nm0 = scratch, *nm1 = scratch + (size_t)ctx->nmoving * ctx->G * ctx->N;
-    return launch_project_nm<T>(ctx, I, Ip, mom, 10, nm0, nm1, st);
+    return launch_project_nm<T>(ctx, I, Ip, mom, nm0, nm1, st);
 }
 
 template cudaError_t launch_project_scratch<double>(const shd_ctx *, const double *, double *, double *, double *,
@@ -1880,8 +1880,8 @@ template cudaError_t launch_project_scratch<float>(const shd_ctx *, const float 
 template cudaError_t launch_moments<double, double>(const shd_ctx *, const double *, double *, cudaStream_t);
 template cudaError_t launch_moments<float, double>(const shd_ctx *, const float *, double *, cudaStream_t);
 template cudaError_t launch_moments<float, float>(const shd_ctx *, const float *, float *, cudaStream_t);
-template cudaError_t launch_project<double>(const shd_ctx *, const double *, double *, double *, int, cudaStream_t);
-template cudaError_t launch_project<float>(const shd_ctx *, const float *, float *, float *, int, cudaStream_t);
+template cudaError_t launch_project<double>(const shd_ctx *, const double *, double *, double *, cudaStream_t);
+template cudaError_t launch_project<float>(const shd_ctx *, const float *, float *, float *, cudaStream_t);
 template cudaError_t launch_sh2lab<double>(const shd_ctx *, const double *, double *, double *, cudaStream_t, bool);
 template cudaError_t launch_sh2lab<float>(const shd_ctx *, const float *, float *, float *, cudaStream_t, bool);
 
