@@ -194,10 +194,30 @@ int ctx_check(shd_ctx *c)
     return SHD_OK;
 }
 
+void drop_graphs(shd_ctx *c);
+
+// Give the FP64 remap tables back (the remaps then compute in place until the
+// flow changes); false when there are none.
+bool release_remap_tables(shd_ctx *c)
+{
+    if (!is_fp64(c) || c->rtab_n == 0) return false;
+    drop_graphs(c);  // captured steps read them
+    for (void *&p : c->d_rtab) dfree(p);
+    c->bytes -= (long long)(2 * c->rtab_n * remap_entry64_bytes());
+    c->rtab_n = 0;
+    c->rtab_valid = false;
+    c->rtab_declined = true;
+    return true;
+}
+
 int dalloc(shd_ctx *c, void **p, size_t bytes, const char *what)
 {
     dfree(*p);
     cudaError_t e = cudaMalloc(p, bytes ? bytes : 16);
+    if (e == cudaErrorMemoryAllocation) {  // rather this than the optional tables
+        cudaGetLastError();
+        if (release_remap_tables(c)) e = cudaMalloc(p, bytes ? bytes : 16);
+    }
     if (e != cudaSuccess) {
         *p = nullptr;
         return fail(SHD_ERR_OOM, "cudaMalloc %s (%zu bytes): %s", what, bytes, cudaGetErrorString(e));
@@ -225,7 +245,7 @@ void drop_sized(shd_ctx *c)
     c->ntiles = 0;
     c->nmoving = 0;
     c->rtab_n = 0;
-    c->rtab_valid = false;
+    c->rtab_valid = c->rtab_declined = false;
     c->fstage_n = 0;
     c->have_fields = c->have_scat = c->have_state = false;
     c->have_theta = false;
@@ -865,16 +885,27 @@ int ensure_remap_tables(shd_ctx *c, cudaStream_t st)
     const size_t n = (size_t)c->nmoving * c->N;
     int rc;
     if (is_fp64(c)) {
-        if (n != c->rtab_n || !c->d_rtab[0] || !c->d_rtab[1]) {
-            c->rtab_n = 0;
-            for (int i = 0; i < 2; ++i)
-                if (dalloc(c, &c->d_rtab[i], n * remap_entry64_bytes(), "remap tables")) {
-                    // no room: the remaps compute in place
-                    dfree(c->d_rtab[0]);
-                    dfree(c->d_rtab[1]);
-                    cudaGetLastError();
-                    return SHD_OK;
-                }
+        if (n != c->rtab_n) {
+            // They save time only, and with few groups are larger than the
+            // intensity (96 bytes a moving node and ordinate, 8 G a node and
+            // ordinate): taken from an eighth of the free memory at most, what
+            // is left being the caller's, and given back when an allocation of
+            // the library's own fails (dalloc).  Else the remaps compute in
+            // place, the same bits in 1.3 to 1.5 times the remaps' time.
+            const size_t bytes = n * remap_entry64_bytes();
+            size_t free_b = 0, total_b = 0;
+            if (c->rtab_declined) return SHD_OK;
+            release_remap_tables(c);  // another flow's
+            c->rtab_declined = true;
+            bool ok = cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && bytes <= free_b / 16;
+            for (int i = 0; i < 2 && ok; ++i) ok = cudaMalloc(&c->d_rtab[i], bytes) == cudaSuccess;
+            if (!ok) {
+                cudaGetLastError();
+                for (void *&p : c->d_rtab) dfree(p);
+                return SHD_OK;
+            }
+            c->rtab_declined = false;
+            c->bytes += (long long)(2 * bytes);
             c->rtab_n = n;
         }
         CK(launch_remap_tables_d(c, c->d_rtab[0], c->d_rtab[1], c->stream), "remap tables");
@@ -1117,9 +1148,9 @@ template <class T>
 int capture_step(shd_ctx *c, int i)
 {
     if (!c->cap_stream) CK(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking), "capture stream");
-    int rt = ensure_remap_tables(c, nullptr);  // built outside the graph, read in place by every replay
+    int rt = ensure_rk_buffers(c);
     if (rt) return rt;
-    if ((rt = ensure_rk_buffers(c))) return rt;
+    if ((rt = ensure_remap_tables(c, nullptr))) return rt;  // built outside the graph, read in place by every replay
     const unsigned long long n0 = shd_launch_count_now();
     void *sp0 = c->d_Sp, *sprev0 = c->d_Sprev;
     const bool valid0 = c->sprev_valid;
@@ -1232,8 +1263,8 @@ int run_steps(shd_ctx *c, int nsteps, cudaStream_t st, bool graphs = false,
               const std::function<int()> *after_source = nullptr)
 {
     if constexpr (sizeof(T) == 4) sched_cache_take(c);
-    if (int rc = ensure_remap_tables(c, st)) return rc;
     if (int rc = ensure_rk_buffers(c)) return rc;
+    if (int rc = ensure_remap_tables(c, st)) return rc;
     if (int rc = ensure_chi_rest<T>(c, st)) return rc;  // before any capture
     for (int s = 0; s < nsteps; ++s) {
         // a replay of the captured step: a step with S_prev, no timing events
@@ -1514,7 +1545,7 @@ int shd_set_fields(shd_ctx *c, const double *alpha0, const double *ne, const dou
     }
     // the remap tables follow the flow in working precision: rebuilt before
     // the next step when it changed
-    if (!c->have_fields || fc.u_changed) c->rtab_valid = false;
+    if (!c->have_fields || fc.u_changed) c->rtab_valid = c->rtab_declined = false;
     // the node tables (and with them the captured step) change only when the
     // set of moving nodes does; new field values are read in place
     if (!c->have_fields || fc.moving_changed) {
