@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(256) k_source(Prob<T> P, const T *__restrict__
 }
 
 // a2 + a5 fused for the stepping path: one warp per node (persistent grid of
-// n_partial CTAs x 8 warps), the node's I_lm staged in the warp's shared
+// the CTAs that fit at once x 8 warps), the node's I_lm staged in the warp's shared
 // tile, K_l in shared memory with rows padded against bank conflicts.  S_p
 // is formed exactly as k_source forms it; while it is written, every thread
 // accumulates in FP64 the residual |S - S_prev|^2, |S|^2 and, from J of the
@@ -1958,9 +1958,7 @@ cudaError_t launch_source_sums(shd_ctx *ctx, const T *Ip, T *Sp, const T *mom, c
     auto kern = ctx->k_diagonal && ctx->G <= 32 ? k_source_sums<T, true> : k_source_sums<T, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    // at least four nodes a warp: every CTA's eight warps pay the FP64
-    // reduction and the staging of K (16^3: 1216 CTAs 24 us in FP32 and 31 in FP64, 128 CTAs 17 and 21)
-    const int nb = (int)std::min<long long>(ctx->n_partial, (ctx->Nc + 31) / 32);
+    const int nb = ctx->n_partial;
     int grid_cc = nb;  // partial-sum rows of the CUDA-core pass
     auto cuda_cores = [&]() -> cudaError_t {
         if constexpr (sizeof(T) == 4) {
@@ -1993,9 +1991,20 @@ cudaError_t launch_source_sums(shd_ctx *ctx, const T *Ip, T *Sp, const T *mom, c
                 return cudaGetLastError();
             }
         }
-        kern<<<nb, 256, sm, st>>>(P, Ip, Sp, mom, Sprev, have_prev ? 1 : 0, ctx->d_partial);
+        // the CTAs that fit at once (every CTA's eight warps pay the FP64
+        // reduction and the staging of K, and fewer leave SMs idle where a node
+        // is much work), a node a warp at least.  16^3, one group, FP64: 1216
+        // CTAs 42 us, 304 31, 128 33; 12^3, 32 groups, FP64: 74, 67, 81 (the
+        // group-mixing kernel 263, 256, 262, and 492 with 54); 48^3, 16 groups,
+        // FP32: 223, 197 (456 CTAs), 525
+        int sms = 0, per_sm = 0;
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess || sms <= 0)
+            sms = 148;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, sm) != cudaSuccess || per_sm < 1)
+            per_sm = 1;
+        grid_cc = (int)std::min<long long>(std::min(nb, sms * per_sm), (ctx->Nc + 7) / 8);
+        kern<<<grid_cc, 256, sm, st>>>(P, Ip, Sp, mom, Sprev, have_prev ? 1 : 0, ctx->d_partial);
         note_launch();
-        grid_cc = nb;
         return cudaGetLastError();
     };
     bool tc = false;
