@@ -371,8 +371,9 @@ unsigned long long shd_launch_count(void);
  *   message names it).
  *   In sweep mode 1 the replayed steps of FP32 backward-Euler
  *   problems with the linear short-characteristics integrator, planes the
- *   one-CTA sweep holds, and no cluster schedule forced or timed more than
- *   3 % faster (shd_get_sweep_schedule) run stages a1-a3 per problem and
+ *   one-CTA sweep holds two rows a thread of (more where their columns fit
+ *   768 threads), and no other schedule forced or timed more than 3 % faster
+ *   (shd_get_sweep_schedule) run stages a1-a3 per problem and
  *   then stage a4 of all of them in one persistent launch per kernel
  *   variant, over a work list of every such problem's (ordinate, group)
  *   pairs; the other problems sweep in their own launches.  Results are

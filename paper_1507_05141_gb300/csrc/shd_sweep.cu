@@ -166,13 +166,24 @@ __device__ __forceinline__ void halo_wait(uint32_t bar, uint32_t parity, bool &d
 // exchange's threads at compile time (0: ns_rt), the ring then NS R + 8 reals
 // an array (else ps_rt); hs_rt: the halo slots' columns.  tune_col >= 0
 // (schedule timing only): into column tune_col of a scratch intensity [.][Nc].
-template <int R, int V, int NS, bool CL, bool FLAT>
-__device__ __forceinline__ void sweep_pair_rays(const Prob<float> &P, float *__restrict__ I,
-                                               const float *__restrict__ eta, const float *__restrict__ chi,
-                                               const float *__restrict__ chi0L,
-                                               const unsigned long long *__restrict__ mbits, int npc, int nwin,
-                                               int pair, long long tune_col, int ps_rt, int ns_rt, int hs_rt,
-                                               bool wide, int *err, unsigned char *smem_raw)
+// MEM: A lies in shared memory and is read again for every plane (a batch's
+// descriptor: its pointers would not fit the registers, where a launch of its
+// own has them as constant operands).
+struct SweepArrays {
+    float *I;
+    const float *eta, *chi, *chi0L;
+    const unsigned long long *mbits;
+};
+template <class Q>
+__device__ __forceinline__ Q array_of(const Q &p)
+{
+    return *const_cast<const volatile Q *>(&p);
+}
+
+template <int R, int V, int NS, bool CL, bool FLAT, bool MEM>
+__device__ __forceinline__ void sweep_pair_rays(const Prob<float> &P, const SweepArrays &A, int npc, int nwin, int pair,
+                                               long long tune_col, int ps_rt, int ns_rt, int hs_rt, bool wide, int *err,
+                                               unsigned char *smem_raw)
 {
     const int k = pair / P.G;
     const int g = pair - k * P.G;
@@ -224,10 +235,29 @@ __device__ __forceinline__ void sweep_pair_rays(const Prob<float> &P, float *__r
     }
     const int nloc = nrows * n2, j0 = row0 * n2;
     const long long base = ((long long)k * P.G + g) * P.Nc;
-    if (tune_col >= 0) I += tune_col * P.Nc - base;
-    const bool table = chi0L != nullptr;
-    const float *c0base = table ? chi0L + ((long long)od * P.G + g) * P.Nc : nullptr;
-    const unsigned long long *mb = table ? mbits + (size_t)od * nwin * npc : nullptr;
+    const bool table = A.chi0L != nullptr;
+    auto I_of = [&, I = MEM ? nullptr : (tune_col >= 0 ? A.I + (tune_col * P.Nc - base) : A.I)]() -> float * {
+        if constexpr (MEM) return array_of(A.I);
+        else return I;
+    };
+    auto eta_of = [&, e = MEM ? nullptr : A.eta]() -> const float * {
+        if constexpr (MEM) return array_of(A.eta);
+        else return e;
+    };
+    auto chi_of = [&, e = MEM ? nullptr : A.chi]() -> const float * {
+        if constexpr (MEM) return array_of(A.chi);
+        else return e;
+    };
+    const long long c0off = ((long long)od * P.G + g) * P.Nc;
+    auto chi0_of = [&, e = MEM || !table ? nullptr : A.chi0L + c0off]() -> const float * {
+        if constexpr (MEM) return array_of(A.chi0L) + c0off;
+        else return e;
+    };
+    const size_t mb0 = (size_t)od * nwin * npc;
+    auto bits_of = [&, e = MEM || !table ? nullptr : A.mbits + mb0]() -> const unsigned long long * {
+        if constexpr (MEM) return array_of(A.mbits) + mb0;
+        else return e;
+    };
     const float fr1 = (float)o.fr1, fr2 = (float)o.fr2, hs = (float)o.s * 0.5f, kap = P.kappa;
     const float w00 = (1.f - fr1) * (1.f - fr2), w10 = fr1 * (1.f - fr2), w01 = (1.f - fr1) * fr2, w11 = fr1 * fr2;
     const float bc_iso = P.bc_mode == SHD_BC_ISO ? P.bc[g] : 0.f;
@@ -271,6 +301,7 @@ __device__ __forceinline__ void sweep_pair_rays(const Prob<float> &P, float *__r
         if (step < nd && nrows > 0) {
             const int id = fwd ? step : nd - 1 - step;
             const long long pb = base + (long long)id * plane + j0;
+            const float *I = I_of(), *eta = eta_of(), *chi = chi_of();
             if (!table) {
                 const int aI = shift16(I + pb), aE = shift16(eta + pb), aC = shift16(chi + pb);
                 const float *gI = I + pb - aI, *gE = eta + pb - aE, *gC = chi + pb - aC;
@@ -282,13 +313,14 @@ __device__ __forceinline__ void sweep_pair_rays(const Prob<float> &P, float *__r
                 const int np = nloc / 4;  // 16-byte pieces per array (aligned planes)
                 if ((id >> 6) != mwin) {
                     mwin = id >> 6;
+                    const unsigned long long *mb = bits_of();
 #pragma unroll
                     for (int i = 0; i < MP; ++i) {
                         const int q = tid + i * nthr;
                         mw[i] = q < np ? mb[(size_t)mwin * npc + (j0 >> 2) + q] : 0ull;
                     }
                 }
-                const float *c0 = c0base + (long long)id * plane + j0;
+                const float *c0 = chi0_of() + (long long)id * plane + j0;
 #pragma unroll
                 for (int i = 0; i < MP; ++i) {
                     const int q = tid + i * nthr;
@@ -324,7 +356,7 @@ __device__ __forceinline__ void sweep_pair_rays(const Prob<float> &P, float *__r
         const long long pb = base + (long long)id * plane + j0;
         // the three arrays share the plane's offset in its aligned cover (when
         // timing, the scratch intensity's may differ: any finite value serves)
-        const float *rI = ring + PAR * 3 * pstride + (table ? 0 : shift16(eta + pb));
+        const float *rI = ring + PAR * 3 * pstride + (table ? 0 : shift16(eta_of() + pb));
         const float *rE = rI + pstride, *rC = rI + 2 * pstride;
         const ColExchange<R> xp{xbuf + (1 - PAR) * xsize, ns}, xn{xbuf + PAR * xsize, ns};
         if constexpr (CL) {
@@ -461,7 +493,7 @@ __device__ __forceinline__ void sweep_pair_rays(const Prob<float> &P, float *__r
                         : "memory");
                 }
             }
-            float *const ig = I + pb;
+            float *const ig = I_of() + pb;
             if (exact) {
 #pragma unroll
                 for (int q = 0; q < R; ++q) ig[off[v][q]] = u[q].x;
@@ -491,20 +523,16 @@ __device__ __forceinline__ void sweep_pair_rays(const Prob<float> &P, float *__r
 // FLAT: the ray has no component along the rows; another row's state, though
 // its weight is 0, must not enter then (it may be infinite).  Code of its own:
 // as a branch in the loop it cost every ray 1.5 to 4 % of the sweep.
-template <int R, int V, int NS, bool CL>
-__device__ __forceinline__ void sweep_pair_col(const Prob<float> &P, float *__restrict__ I,
-                                               const float *__restrict__ eta, const float *__restrict__ chi,
-                                               const float *__restrict__ chi0L,
-                                               const unsigned long long *__restrict__ mbits, int npc, int nwin,
-                                               int pair, long long tune_col, int ps_rt, int ns_rt, int hs_rt,
-                                               bool wide, int *err, unsigned char *smem_raw)
+template <int R, int V, int NS, bool CL, bool MEM = false>
+__device__ __forceinline__ void sweep_pair_col(const Prob<float> &P, const SweepArrays &A, int npc, int nwin, int pair,
+                                               long long tune_col, int ps_rt, int ns_rt, int hs_rt, bool wide, int *err,
+                                               unsigned char *smem_raw)
 {
     if (P.ord[pair / P.G].s1 == 0)
-        sweep_pair_rays<R, V, NS, CL, true>(P, I, eta, chi, chi0L, mbits, npc, nwin, pair, tune_col, ps_rt, ns_rt, hs_rt,
-                                            wide, err, smem_raw);
+        sweep_pair_rays<R, V, NS, CL, true, MEM>(P, A, npc, nwin, pair, tune_col, ps_rt, ns_rt, hs_rt, wide, err, smem_raw);
     else
-        sweep_pair_rays<R, V, NS, CL, false>(P, I, eta, chi, chi0L, mbits, npc, nwin, pair, tune_col, ps_rt, ns_rt,
-                                             hs_rt, wide, err, smem_raw);
+        sweep_pair_rays<R, V, NS, CL, false, MEM>(P, A, npc, nwin, pair, tune_col, ps_rt, ns_rt, hs_rt, wide, err,
+                                                  smem_raw);
 }
 
 // One CTA a plane.  NT bounds the threads (the launch takes as many as the
@@ -526,7 +554,7 @@ __global__ void __launch_bounds__(NT, col_min_ctas(NT, R)) k_sweep_col(Prob<floa
     // tune_stride > 0 (schedule timing only): CTA b sweeps pair b * tune_stride
     // with its intensity in column b of a scratch array I [b][Nc]
     const int pair = tune_stride > 0 ? (int)blockIdx.x * tune_stride : (int)blockIdx.x;
-    sweep_pair_col<R, V, NS, false>(P, I, eta, chi, chi0L, mbits, npc, nwin, pair,
+    sweep_pair_col<R, V, NS, false>(P, SweepArrays{I, eta, chi, chi0L, mbits}, npc, nwin, pair,
                                                  tune_stride > 0 ? (long long)blockIdx.x : -1, pstride, ns, hs,
                                                  wide != 0, err, smem_raw);
 }
@@ -542,7 +570,7 @@ __global__ void __launch_bounds__(NT, col_min_ctas(NT, R)) k_sweep_cl(Prob<float
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int cidx = (int)blockIdx.x / (int)cg::this_cluster().num_blocks();
     const int pair = tune_stride > 0 ? cidx * tune_stride : cidx;
-    sweep_pair_col<R, V, NS, true>(P, I, eta, chi, chi0L, mbits, npc, nwin, pair,
+    sweep_pair_col<R, V, NS, true>(P, SweepArrays{I, eta, chi, chi0L, mbits}, npc, nwin, pair,
                                                 tune_stride > 0 ? (long long)cidx : -1, pstride, ns, hs, wide != 0,
                                                 err, smem_raw);
 }
@@ -551,12 +579,13 @@ __global__ void __launch_bounds__(NT, col_min_ctas(NT, R)) k_sweep_cl(Prob<float
 // walk the work list of every problem's (ordinate, group) pairs (problem p
 // owns items [item0, item0 + N G)), each item as k_sweep_col sweeps it, with
 // the problem's own fields and arrays.  One launch per class of problems
-// that share the rows a thread holds (R).
-template <int R>
-__global__ void __launch_bounds__(1024, 1) k_sweep_batch(const SweepBatchProb *__restrict__ bp, int nprob,
+// that share the kernel's variant.
+template <int R, int NT, int NS>
+__global__ void __launch_bounds__(NT, col_min_ctas(NT, R)) k_sweep_batch(const SweepBatchProb *__restrict__ bp, int nprob,
                                                          long long nitems)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ SweepArrays A;
     for (long long it = blockIdx.x; it < nitems; it += gridDim.x) {
         int lo = 0, hi = nprob - 1;  // the last problem whose first item is <= it
         while (lo < hi) {
@@ -566,8 +595,10 @@ __global__ void __launch_bounds__(1024, 1) k_sweep_batch(const SweepBatchProb *_
         }
         const SweepBatchProb &b = bp[lo];
         __syncthreads();  // the previous item's reads of the shared buffers are done
-        sweep_pair_col<R, 1, 0, false>(b.P, b.I, b.eta, b.chi, b.chi0L, b.mbits, b.npc, b.nwin,
-                                       (int)(it - b.item0), -1, b.pstride, b.ns, 0, b.wide != 0, nullptr, smem_raw);
+        if (threadIdx.x == 0) A = SweepArrays{b.I, b.eta, b.chi, b.chi0L, b.mbits};
+        __syncthreads();
+        sweep_pair_col<R, 1, NS, false, true>(b.P, A, b.npc, b.nwin, (int)(it - b.item0), -1, b.pstride, b.ns, 0,
+                                              b.wide != 0, nullptr, smem_raw);
     }
 }
 
@@ -636,9 +667,8 @@ static int sweep_columns(const shd_ctx *c)
 }
 
 // R, V, the thread bound of the kernel, the buffers of schedule (C, NT):
-// strides at compile time for R <= 4 where they fit (batch: never), else at
-// run time
-static bool sweep_plan(const shd_ctx *c, SweepSched &sc, bool batch = false)
+// strides at compile time for R <= 4 where they fit, else at run time
+static bool sweep_plan(const shd_ctx *c, SweepSched &sc)
 {
     const size_t limit = 227 * 1024;
     const int ps = ((sweep_nloc_max(c, sc.C) + 3) & ~3) + (sc.C == 1 ? 4 : 0);
@@ -651,8 +681,8 @@ static bool sweep_plan(const shd_ctx *c, SweepSched &sc, bool batch = false)
         const int nthr = ((slots + V - 1) / V + 31) & ~31;
         // one CTA a plane of 513 to 768 threads: the kernel bounded by 768,
         // with 85 registers a thread instead of 64
-        const int cap = !batch && sc.C == 1 && sc.NT == 1024 && V == 1 && R <= 6 && nthr > 512 && nthr <= 768 ? 768 : sc.NT;
-        for (int rt = batch || R > 4 || V > 1; rt < (batch || R > 2 || V > 1 ? 2 : 1); ++rt) {
+        const int cap = sc.C == 1 && sc.NT == 1024 && V == 1 && R <= 6 && nthr > 512 && nthr <= 768 ? 768 : sc.NT;
+        for (int rt = R > 4 || V > 1; rt < (R > 2 || V > 1 ? 2 : 1); ++rt) {
             sc.ns = rt ? (slots + 3) & ~3 : cap * V;
             sc.pstride = rt ? ps : cap * V * R + 8;
             sc.hs = sc.C > 1 ? sweep_columns(c) : 0;
@@ -872,11 +902,17 @@ static bool sweep_schedule(const shd_ctx *cc, cudaStream_t st, const float *eta,
 }
 
 // ---- the batch's sweep ----------------------------------------------------------
+// A batch's launch sweeps the problems that the one-CTA schedule of 1024
+// threads sweeps, with the variant that their own launch of it takes
+// (k_sweep_col's R and thread bound; one variant an R with strides at run time
+// was slower than the node-a-thread kernel before it: four 48^3 jets, 12
+// groups, 20.8 ms a step then, 23.0 with it, 18.8 now).  Variants of more than
+// two rows under the 64 registers of 1024 threads spill without a launch's
+// constant operands (three 64^3 jets 23.6 ms, 19.3 in launches of their own,
+// 22.5 before; 52^3 19.3, 15.8, 17.9): those problems sweep on their own.
 static bool sweep_batch_plan(const shd_ctx *c, SweepSched &sc)
 {
-    if (!sweep_sched_make(c, 1, 1024, sc)) return false;
-    sc.R = 0;
-    return sweep_plan(c, sc, true) && sc.V == 1;
+    return sweep_sched_make(c, 1, 1024, sc) && sc.R > 0 && sc.V == 1 && !sc.rt && (sc.R <= 2 || sc.cap == 768);
 }
 
 size_t sweep_batch_smem(const shd_ctx *c)
@@ -921,7 +957,7 @@ int sweep_batch_class(const shd_ctx *c)
         }
         if (!(pp > 0.f && pp <= 1.03f * best)) return 0;
     }
-    return sc.R;
+    return sc.R * 8 + sc.cap / 256;
 }
 
 cudaError_t launch_sweep_batch(int cls, const SweepBatchProb *d_probs, int nprob, long long nitems, size_t smem,
@@ -930,23 +966,24 @@ cudaError_t launch_sweep_batch(int cls, const SweepBatchProb *d_probs, int nprob
     if (nprob <= 0 || nitems <= 0) return cudaSuccess;
     using KB = void (*)(const SweepBatchProb *, int, long long);
     KB kern = nullptr;
+    int NT = 1024;
     switch (cls) {
-        case 1: kern = k_sweep_batch<1>; break;
-        case 2: kern = k_sweep_batch<2>; break;
-        case 3: kern = k_sweep_batch<3>; break;
-        case 4: kern = k_sweep_batch<4>; break;
-        case 6: kern = k_sweep_batch<6>; break;
-        case 8: kern = k_sweep_batch<8>; break;
+        case 1 * 8 + 3: kern = k_sweep_batch<1, 768, 768>, NT = 768; break;
+        case 1 * 8 + 4: kern = k_sweep_batch<1, 1024, 1024>; break;
+        case 2 * 8 + 3: kern = k_sweep_batch<2, 768, 768>, NT = 768; break;
+        case 2 * 8 + 4: kern = k_sweep_batch<2, 1024, 1024>; break;
+        case 3 * 8 + 3: kern = k_sweep_batch<3, 768, 768>, NT = 768; break;
+        case 4 * 8 + 3: kern = k_sweep_batch<4, 768, 768>, NT = 768; break;
         default: return cudaErrorInvalidConfiguration;
     }
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int nsm = 0, per = 0;
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || nsm <= 0) nsm = 148;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, 1024, smem) != cudaSuccess || per < 1) per = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, NT, smem) != cudaSuccess || per < 1) per = 1;
     long long grid = (long long)nsm * per;  // persistent: every CTA that fits at once
     if (grid > nitems) grid = nitems;
-    kern<<<(unsigned)grid, 1024, smem, st>>>(d_probs, nprob, nitems);
+    kern<<<(unsigned)grid, NT, smem, st>>>(d_probs, nprob, nitems);
     note_launch();
     return cudaGetLastError();
 }
