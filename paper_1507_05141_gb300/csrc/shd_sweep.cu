@@ -133,7 +133,7 @@ struct ColExchange {
 };
 
 // ---- the cluster's halo channel --------------------------------------------
-constexpr int kHaloSlots = 4;
+constexpr int kHaloShift = 2;  // log2 of the slots: 4, or 2 where the planes' columns leave no room for them
 constexpr long long kHaloWaitLimit = 1LL << 22;  // mbarrier polls before giving up (about a second)
 
 __device__ __forceinline__ uint32_t remote_addr(uint32_t local, int rank)
@@ -164,7 +164,8 @@ __device__ __forceinline__ void halo_wait(uint32_t bar, uint32_t parity, bool &d
 // One (ordinate, group) pair.  V: column passes of a plane with more columns
 // than threads (thread t also plays threads t + blockDim.x, ...).  NS: the
 // exchange's threads at compile time (0: ns_rt), the ring then NS R + 8 reals
-// an array (else ps_rt); hs_rt: the halo slots' columns.  tune_col >= 0
+// an array (else ps_rt); hs_rt: the halo slots' columns, hsh_rt: log2 of their
+// number (NS: kHaloShift).  tune_col >= 0
 // (schedule timing only): into column tune_col of a scratch intensity [.][Nc].
 // MEM: A lies in shared memory and is read again for every plane (a batch's
 // descriptor: its pointers would not fit the registers, where a launch of its
@@ -182,8 +183,8 @@ __device__ __forceinline__ Q array_of(const Q &p)
 
 template <int R, int V, int NS, bool CL, bool FLAT, bool MEM>
 __device__ __forceinline__ void sweep_pair_rays(const Prob<float> &P, const SweepArrays &A, int npc, int nwin, int pair,
-                                               long long tune_col, int ps_rt, int ns_rt, int hs_rt, bool wide, int *err,
-                                               unsigned char *smem_raw)
+                                               long long tune_col, int ps_rt, int ns_rt, int hs_rt, int hsh_rt, bool wide,
+                                               int *err, unsigned char *smem_raw)
 {
     const int k = pair / P.G;
     const int g = pair - k * P.G;
@@ -198,9 +199,10 @@ __device__ __forceinline__ void sweep_pair_rays(const Prob<float> &P, const Swee
     const int xsize = ns * ColExchange<R>::kReals;
     float *const ring = reinterpret_cast<float *>(smem_raw);  // [2][3][pstride]
     float *const xbuf = ring + 6 * pstride;                   // [2][xsize]
-    // cluster: halo slots [kHaloSlots][hs] float4, then full and free barriers
+    // cluster: halo slots [slots][hs] float4, then full and free barriers
+    const int hsh = NS ? kHaloShift : hsh_rt, slots = 1 << hsh;
     float4 *const halo = reinterpret_cast<float4 *>(xbuf + 2 * xsize);
-    uint64_t *const hbar = reinterpret_cast<uint64_t *>(halo + kHaloSlots * hs_rt);
+    uint64_t *const hbar = reinterpret_cast<uint64_t *>(halo + slots * hs_rt);
     // this CTA's rows
     int row0 = 0, nrows = n1, up = -1, down = -1;
     if constexpr (CL) {
@@ -220,12 +222,12 @@ __device__ __forceinline__ void sweep_pair_rays(const Prob<float> &P, const Swee
             if (down < 0 || down >= used) down = -1;
         }
         if (tid == 0) {
-            for (int i = 0; i < 2 * kHaloSlots; ++i)
+            for (int i = 0; i < 2 * slots; ++i)
                 asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"((uint32_t)__cvta_generic_to_shared(hbar + i))
                              : "memory");
             asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
             if (up >= 0)
-                for (int i = 0; i < kHaloSlots; ++i)
+                for (int i = 0; i < slots; ++i)
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(
                                      (uint32_t)__cvta_generic_to_shared(hbar + i)),
                                  "r"(16 * n2)
@@ -362,14 +364,14 @@ __device__ __forceinline__ void sweep_pair_rays(const Prob<float> &P, const Swee
         if constexpr (CL) {
             // the reads of halo slot step - 2 are done: hand it back
             if (up >= 0 && tid == 0 && step >= 2) {
-                const int h = (step - 2) & (kHaloSlots - 1);
-                if (step - 2 + kHaloSlots <= nd - 2) {
+                const int h = (step - 2) & (slots - 1);
+                if (step - 2 + slots <= nd - 2) {
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(
                                      (uint32_t)__cvta_generic_to_shared(hbar + h)),
                                  "r"(16 * n2)
                                  : "memory");
                     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];\n" ::"r"(
-                                     remote_addr((uint32_t)__cvta_generic_to_shared(hbar + kHaloSlots + h), up))
+                                     remote_addr((uint32_t)__cvta_generic_to_shared(hbar + slots + h), up))
                                  : "memory");
                 }
             }
@@ -388,9 +390,9 @@ __device__ __forceinline__ void sweep_pair_rays(const Prob<float> &P, const Swee
                 float hac = 0.f, hbc = 0.f;
                 if constexpr (!FLAT) {
                     if (CL && first_rb[v]) {
-                        const int h = (step - 1) & (kHaloSlots - 1);
+                        const int h = (step - 1) & (slots - 1);
                         halo_wait((uint32_t)__cvta_generic_to_shared(hbar + h),
-                                  (uint32_t)(((step - 1) / kHaloSlots) & 1), dead, err);
+                                  (uint32_t)(((step - 1) >> hsh) & 1), dead, err);
                         const float4 A = halo[h * hs_rt + t], B = halo[h * hs_rt + slot_n[v]];
                         ha = make_float2(A.x, A.y);
                         hac = A.z;
@@ -481,10 +483,10 @@ __device__ __forceinline__ void sweep_pair_rays(const Prob<float> &P, const Swee
                         }
                 }
                 if (step <= nd - 2) {
-                    const int h = step & (kHaloSlots - 1);
-                    if (step >= kHaloSlots)
-                        halo_wait((uint32_t)__cvta_generic_to_shared(hbar + kHaloSlots + h),
-                                  (uint32_t)((step / kHaloSlots - 1) & 1), dead, err);
+                    const int h = step & (slots - 1);
+                    if (step >= slots)
+                        halo_wait((uint32_t)__cvta_generic_to_shared(hbar + slots + h),
+                                  (uint32_t)(((step >> hsh) - 1) & 1), dead, err);
                     asm volatile(
                         "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];\n" ::"r"(
                             remote_addr((uint32_t)__cvta_generic_to_shared(halo + h * hs_rt + t - (nb - 1) * n2), down)),
@@ -525,13 +527,14 @@ __device__ __forceinline__ void sweep_pair_rays(const Prob<float> &P, const Swee
 // as a branch in the loop it cost every ray 1.5 to 4 % of the sweep.
 template <int R, int V, int NS, bool CL, bool MEM = false>
 __device__ __forceinline__ void sweep_pair_col(const Prob<float> &P, const SweepArrays &A, int npc, int nwin, int pair,
-                                               long long tune_col, int ps_rt, int ns_rt, int hs_rt, bool wide, int *err,
-                                               unsigned char *smem_raw)
+                                               long long tune_col, int ps_rt, int ns_rt, int hs_rt, int hsh_rt, bool wide,
+                                               int *err, unsigned char *smem_raw)
 {
     if (P.ord[pair / P.G].s1 == 0)
-        sweep_pair_rays<R, V, NS, CL, true, MEM>(P, A, npc, nwin, pair, tune_col, ps_rt, ns_rt, hs_rt, wide, err, smem_raw);
+        sweep_pair_rays<R, V, NS, CL, true, MEM>(P, A, npc, nwin, pair, tune_col, ps_rt, ns_rt, hs_rt, hsh_rt, wide, err,
+                                                 smem_raw);
     else
-        sweep_pair_rays<R, V, NS, CL, false, MEM>(P, A, npc, nwin, pair, tune_col, ps_rt, ns_rt, hs_rt, wide, err,
+        sweep_pair_rays<R, V, NS, CL, false, MEM>(P, A, npc, nwin, pair, tune_col, ps_rt, ns_rt, hs_rt, hsh_rt, wide, err,
                                                   smem_raw);
 }
 
@@ -548,14 +551,14 @@ __global__ void __launch_bounds__(NT, col_min_ctas(NT, R)) k_sweep_col(Prob<floa
                                                    const float *__restrict__ eta, const float *__restrict__ chi,
                                                    const float *__restrict__ chi0L,
                                                    const unsigned long long *__restrict__ mbits, int npc, int nwin,
-                                                   int pstride, int ns, int hs, int wide, int *err, int tune_stride)
+                                                   int pstride, int ns, int hs, int hsh, int wide, int *err, int tune_stride)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     // tune_stride > 0 (schedule timing only): CTA b sweeps pair b * tune_stride
     // with its intensity in column b of a scratch array I [b][Nc]
     const int pair = tune_stride > 0 ? (int)blockIdx.x * tune_stride : (int)blockIdx.x;
     sweep_pair_col<R, V, NS, false>(P, SweepArrays{I, eta, chi, chi0L, mbits}, npc, nwin, pair,
-                                                 tune_stride > 0 ? (long long)blockIdx.x : -1, pstride, ns, hs,
+                                                 tune_stride > 0 ? (long long)blockIdx.x : -1, pstride, ns, hs, hsh,
                                                  wide != 0, err, smem_raw);
 }
 
@@ -565,13 +568,13 @@ __global__ void __launch_bounds__(NT, col_min_ctas(NT, R)) k_sweep_cl(Prob<float
                                                    const float *__restrict__ eta, const float *__restrict__ chi,
                                                    const float *__restrict__ chi0L,
                                                    const unsigned long long *__restrict__ mbits, int npc, int nwin,
-                                                   int pstride, int ns, int hs, int wide, int *err, int tune_stride)
+                                                   int pstride, int ns, int hs, int hsh, int wide, int *err, int tune_stride)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int cidx = (int)blockIdx.x / (int)cg::this_cluster().num_blocks();
     const int pair = tune_stride > 0 ? cidx * tune_stride : cidx;
     sweep_pair_col<R, V, NS, true>(P, SweepArrays{I, eta, chi, chi0L, mbits}, npc, nwin, pair,
-                                                tune_stride > 0 ? (long long)cidx : -1, pstride, ns, hs, wide != 0,
+                                                tune_stride > 0 ? (long long)cidx : -1, pstride, ns, hs, hsh, wide != 0,
                                                 err, smem_raw);
 }
 
@@ -597,7 +600,7 @@ __global__ void __launch_bounds__(NT, col_min_ctas(NT, R)) k_sweep_batch(const S
         __syncthreads();  // the previous item's reads of the shared buffers are done
         if (threadIdx.x == 0) A = SweepArrays{b.I, b.eta, b.chi, b.chi0L, b.mbits};
         __syncthreads();
-        sweep_pair_col<R, 1, NS, false, true>(b.P, A, b.npc, b.nwin, (int)(it - b.item0), -1, b.pstride, b.ns, 0,
+        sweep_pair_col<R, 1, NS, false, true>(b.P, A, b.npc, b.nwin, (int)(it - b.item0), -1, b.pstride, b.ns, 0, 0,
                                               b.wide != 0, nullptr, smem_raw);
     }
 }
@@ -612,9 +615,9 @@ __global__ void __launch_bounds__(NT, col_min_ctas(NT, R)) k_sweep_batch(const S
 
 struct SweepSched {
     int C = 0, NT = 0;
-    int R = 0, V = 0, cap = 0, nthr = 0;  // R = 0: none fits (the generic sweep)
+    int R = 0, V = 0, cap = 0, nthr = 0;
     bool rt = false;                      // strides at run time
-    int pstride = 0, ns = 0, hs = 0;
+    int pstride = 0, ns = 0, hs = 0, hsh = 0;
     size_t smem = 0;
 };
 
@@ -667,41 +670,45 @@ static int sweep_columns(const shd_ctx *c)
 }
 
 // R, V, the thread bound of the kernel, the buffers of schedule (C, NT):
-// strides at compile time for R <= 4 where they fit, else at run time
+// strides at compile time for R <= 4 where they fit, else at run time; two
+// halo slots only where four leave no plan (planes of some 800 columns and
+// more).  Not built: one row a thread in a cluster (blocks of at most NT nodes
+// run two rows on half the threads) and eight rows below 1024 threads.
 static bool sweep_plan(const shd_ctx *c, SweepSched &sc)
 {
     const size_t limit = 227 * 1024;
     const int ps = ((sweep_nloc_max(c, sc.C) + 3) & ~3) + (sc.C == 1 ? 4 : 0);
     static const int Rs[7] = {1, 2, 3, 4, 6, 8, 1}, Vs[7] = {1, 1, 1, 1, 1, 1, 4};
-    for (int i = 0; i < 7; ++i) {
-        const int R = Rs[i], V = Vs[i];
-        if ((R == 8 && sc.NT != 1024) || (R == 1 && V == 1 && sc.C > 1)) continue;
-        const int slots = sweep_threads(c, sc.C, R);
-        if (slots > sc.NT * V) continue;
-        const int nthr = ((slots + V - 1) / V + 31) & ~31;
-        // one CTA a plane of 513 to 768 threads: the kernel bounded by 768,
-        // with 85 registers a thread instead of 64
-        const int cap = sc.C == 1 && sc.NT == 1024 && V == 1 && R <= 6 && nthr > 512 && nthr <= 768 ? 768 : sc.NT;
-        for (int rt = R > 4 || V > 1; rt < (R > 2 || V > 1 ? 2 : 1); ++rt) {
-            sc.ns = rt ? (slots + 3) & ~3 : cap * V;
-            sc.pstride = rt ? ps : cap * V * R + 8;
-            sc.hs = sc.C > 1 ? sweep_columns(c) : 0;
-            sc.smem = sizeof(float) * (6 * (size_t)sc.pstride + 2 * (size_t)sc.ns * 3 * R) +
-                      (sc.C > 1 ? (size_t)kHaloSlots * (16 * (size_t)sc.hs + 16) : 0);
-            if (sc.pstride < ps || sc.smem > limit) continue;
-            sc.R = R;
-            sc.V = V;
-            sc.rt = rt != 0;
-            sc.nthr = nthr;
-            sc.cap = cap;
-            return true;
+    sc.hs = sc.C > 1 ? sweep_columns(c) : 0;
+    for (sc.hsh = kHaloShift; sc.hsh >= (sc.C > 1 ? 1 : kHaloShift); --sc.hsh)
+        for (int i = 0; i < 7; ++i) {
+            const int R = Rs[i], V = Vs[i];
+            if ((R == 8 && sc.NT != 1024) || (R == 1 && V == 1 && sc.C > 1)) continue;
+            const int slots = sweep_threads(c, sc.C, R);
+            if (slots > sc.NT * V) continue;
+            const int nthr = ((slots + V - 1) / V + 31) & ~31;
+            // one CTA a plane of 513 to 768 threads: the kernel bounded by 768,
+            // with 85 registers a thread instead of 64
+            const int cap = sc.C == 1 && sc.NT == 1024 && V == 1 && R <= 6 && nthr > 512 && nthr <= 768 ? 768 : sc.NT;
+            for (int rt = R > 4 || V > 1 || sc.hsh != kHaloShift; rt < (R > 2 || V > 1 ? 2 : 1); ++rt) {
+                sc.ns = rt ? (slots + 3) & ~3 : cap * V;
+                sc.pstride = rt ? ps : cap * V * R + 8;
+                sc.smem = sizeof(float) * (6 * (size_t)sc.pstride + 2 * (size_t)sc.ns * 3 * R) +
+                          (sc.C > 1 ? ((size_t)1 << sc.hsh) * (16 * (size_t)sc.hs + 16) : 0);
+                if (sc.pstride < ps || sc.smem > limit) continue;
+                sc.R = R;
+                sc.V = V;
+                sc.rt = rt != 0;
+                sc.nthr = nthr;
+                sc.cap = cap;
+                return true;
+            }
         }
-    }
     return false;
 }
 
 using SweepKernel = void (*)(Prob<float>, float *, const float *, const float *, const float *,
-                             const unsigned long long *, int, int, int, int, int, int, int *, int);
+                             const unsigned long long *, int, int, int, int, int, int, int, int *, int);
 
 template <int R, int V, int NT, int NS, bool CL>
 static SweepKernel sweep_kernel_of()
@@ -778,7 +785,7 @@ static cudaError_t run_sweep_sched(const shd_ctx *ctx, const SweepSched &sc, flo
     cfg.attrs = at;
     cfg.numAttrs = sc.C > 1 ? 1 : 0;
     e = cudaLaunchKernelEx(&cfg, kern, P, I, eta, chi, c0L, mb, ctx->mbits_npc, ctx->mbits_nwin, sc.pstride, sc.ns, sc.hs,
-                           wide ? 1 : 0, ctx->d_tc_err, tune_stride);
+                           sc.hsh, wide ? 1 : 0, ctx->d_tc_err, tune_stride);
     note_launch();
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
@@ -807,8 +814,7 @@ static bool sweep_sched_make(const shd_ctx *c, int C, int NT, SweepSched &sc)
     }
     sc.C = C;
     sc.NT = NT;
-    sweep_plan(c, sc);
-    return true;
+    return sweep_plan(c, sc);  // (every schedule of these bounds has one)
 }
 
 // Every schedule that fits, one CTA a plane first.
@@ -817,10 +823,10 @@ static std::vector<SweepSched> sweep_candidates(const shd_ctx *c, size_t most = 
     std::vector<SweepSched> v;
     SweepSched sc;
     for (int NT : {1024, 512, 256})
-        if (v.size() < most && sweep_sched_make(c, 1, NT, sc) && sc.R) v.push_back(sc);
+        if (v.size() < most && sweep_sched_make(c, 1, NT, sc)) v.push_back(sc);
     for (int C : {2, 4, 8, 16})
         for (int NT : {256, 384, 512, 768, 1024})
-            if (v.size() < most && sweep_sched_make(c, C, NT, sc) && sc.R) v.push_back(sc);
+            if (v.size() < most && sweep_sched_make(c, C, NT, sc)) v.push_back(sc);
     return v;
 }
 
@@ -828,7 +834,7 @@ static std::vector<SweepSched> sweep_candidates(const shd_ctx *c, size_t most = 
 bool sweep_has_schedule(const shd_ctx *c)
 {
     SweepSched sc;
-    if (c->sweep_force_C > 0) return sweep_sched_make(c, c->sweep_force_C, c->sweep_force_NT, sc) && sc.R;
+    if (c->sweep_force_C > 0) return sweep_sched_make(c, c->sweep_force_C, c->sweep_force_NT, sc);
     return !sweep_candidates(c, 1).empty();
 }
 
@@ -840,9 +846,8 @@ static bool sweep_schedule(const shd_ctx *cc, cudaStream_t st, const float *eta,
                            bool wide, SweepSched &out)
 {
     shd_ctx *c = const_cast<shd_ctx *>(cc);  // the choice is a cache of the context
-    // (a forced schedule without a plan runs as the generic sweep)
-    if (c->sweep_force_C > 0) return sweep_sched_make(c, c->sweep_force_C, c->sweep_force_NT, out) && out.R;
-    if (c->sweep_C > 0 && sweep_sched_make(c, c->sweep_C, c->sweep_NT, out) && out.R) return true;
+    if (c->sweep_force_C > 0) return sweep_sched_make(c, c->sweep_force_C, c->sweep_force_NT, out);
+    if (c->sweep_C > 0 && sweep_sched_make(c, c->sweep_C, c->sweep_NT, out)) return true;
     std::vector<SweepSched> cand = sweep_candidates(c);
     if (cand.empty()) return false;
     out = cand[0];
@@ -912,7 +917,7 @@ static bool sweep_schedule(const shd_ctx *cc, cudaStream_t st, const float *eta,
 // 22.5 before; 52^3 19.3, 15.8, 17.9): those problems sweep on their own.
 static bool sweep_batch_plan(const shd_ctx *c, SweepSched &sc)
 {
-    return sweep_sched_make(c, 1, 1024, sc) && sc.R > 0 && sc.V == 1 && !sc.rt && (sc.R <= 2 || sc.cap == 768);
+    return sweep_sched_make(c, 1, 1024, sc) && sc.V == 1 && !sc.rt && (sc.R <= 2 || sc.cap == 768);
 }
 
 size_t sweep_batch_smem(const shd_ctx *c)
