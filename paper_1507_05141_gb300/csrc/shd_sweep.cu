@@ -551,14 +551,16 @@ __global__ void __launch_bounds__(NT, col_min_ctas(NT, R)) k_sweep_col(Prob<floa
                                                    const float *__restrict__ eta, const float *__restrict__ chi,
                                                    const float *__restrict__ chi0L,
                                                    const unsigned long long *__restrict__ mbits, int npc, int nwin,
-                                                   int pstride, int ns, int hs, int hsh, int wide, int *err, int tune_stride)
+                                                   int pstride, int ns, int hs, int hsh, int wide, int *err, int first,
+                                                   int tune_stride)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    // tune_stride > 0 (schedule timing only): CTA b sweeps pair b * tune_stride
-    // with its intensity in column b of a scratch array I [b][Nc]
-    const int pair = tune_stride > 0 ? (int)blockIdx.x * tune_stride : (int)blockIdx.x;
+    // CTA b sweeps pair first + b; with tune_stride > 0 (schedule timing only)
+    // pair (first + b) * tune_stride, its intensity in that column of a scratch
+    // array I [.][Nc]
+    const int idx = first + (int)blockIdx.x, pair = tune_stride > 0 ? idx * tune_stride : idx;
     sweep_pair_col<R, V, NS, false>(P, SweepArrays{I, eta, chi, chi0L, mbits}, npc, nwin, pair,
-                                                 tune_stride > 0 ? (long long)blockIdx.x : -1, pstride, ns, hs, hsh,
+                                                 tune_stride > 0 ? (long long)idx : -1, pstride, ns, hs, hsh,
                                                  wide != 0, err, smem_raw);
 }
 
@@ -568,13 +570,14 @@ __global__ void __launch_bounds__(NT, col_min_ctas(NT, R)) k_sweep_cl(Prob<float
                                                    const float *__restrict__ eta, const float *__restrict__ chi,
                                                    const float *__restrict__ chi0L,
                                                    const unsigned long long *__restrict__ mbits, int npc, int nwin,
-                                                   int pstride, int ns, int hs, int hsh, int wide, int *err, int tune_stride)
+                                                   int pstride, int ns, int hs, int hsh, int wide, int *err, int first,
+                                                   int tune_stride)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int cidx = (int)blockIdx.x / (int)cg::this_cluster().num_blocks();
-    const int pair = tune_stride > 0 ? cidx * tune_stride : cidx;
+    const int idx = first + (int)blockIdx.x / (int)cg::this_cluster().num_blocks();
+    const int pair = tune_stride > 0 ? idx * tune_stride : idx;
     sweep_pair_col<R, V, NS, true>(P, SweepArrays{I, eta, chi, chi0L, mbits}, npc, nwin, pair,
-                                                tune_stride > 0 ? (long long)cidx : -1, pstride, ns, hs, hsh, wide != 0,
+                                                tune_stride > 0 ? (long long)idx : -1, pstride, ns, hs, hsh, wide != 0,
                                                 err, smem_raw);
 }
 
@@ -607,18 +610,26 @@ __global__ void __launch_bounds__(NT, col_min_ctas(NT, R)) k_sweep_batch(const S
 
 // ---- schedules ---------------------------------------------------------------
 // A schedule (C, NT) splits every plane over a cluster of C CTAs of up to NT
-// threads (C = 1: one CTA a plane, k_sweep_col).  Its kernel holds R rows of
-// V columns a thread: R is the least for which the columns of every class's
-// planes fit NT threads (n2 ceil(rows / R) of them); planes with more columns
-// than threads take V = 4 columns of one row.  The launch takes only the
-// threads the largest class needs.
-
-struct SweepSched {
-    int C = 0, NT = 0;
+// threads (C = 1: one CTA a plane, k_sweep_col).  A kernel holds R rows of V
+// columns a thread: R is the least for which the columns of the planes fit NT
+// threads (n2 ceil(rows / R) of them); planes with more columns than threads
+// take V = 4 columns of one row.  The launch takes only the threads the largest
+// plane needs.  One launch sweeps every class of ordinates; where the largest
+// class's planes need a kernel with its strides at run time (many rows a
+// thread above all, which leave the small planes of an elongated grid to a few
+// threads' serial work), classes that need another R or V have launches of
+// their own (8 x 584 x 28, 4 groups, L = 3, 4 CTAs: 2.38 ms a sweep, 8.75 in one
+// launch, 3.08 for the node-a-thread kernel; 8 x 160 x 100: 0.76, 4.43, 1.80).
+struct SweepPart {
+    int k0 = 0, k1 = 0;  // ordinates
     int R = 0, V = 0, cap = 0, nthr = 0;
-    bool rt = false;                      // strides at run time
+    bool rt = false;  // strides at run time
     int pstride = 0, ns = 0, hs = 0, hsh = 0;
     size_t smem = 0;
+};
+struct SweepSched {
+    int C = 0, NT = 0, nparts = 0;
+    SweepPart part[3];
 };
 
 // rows of a plane per CTA of a C-CTA cluster (the kernel's own rule)
@@ -629,32 +640,35 @@ static int sweep_rows_per_cta(int n1, int n2, int C)
     return (R + q4 - 1) / q4 * q4;
 }
 
-// f(n1, n2) for the plane (rows, columns) of each ordinate class present
+// f(n1, n2, first ordinate, end) for the plane (rows, columns) of each ordinate
+// class present in `classes` (bits: z, y, x, their order)
+constexpr int kAllClasses = 7;
 template <class F>
-static void each_plane(const shd_ctx *c, F f)
+static void each_plane(const shd_ctx *c, int classes, F f)
 {
     const int dims[3] = {c->nx, c->ny, c->nz};
-    const int from[3] = {0, c->nZ, c->nA}, to[3] = {c->nZ, c->nA, c->N};  // z, y, x classes
+    const int from[3] = {0, c->nZ, c->nA}, to[3] = {c->nZ, c->nA, c->N};
     for (int i = 0; i < 3; ++i)
-        if (to[i] > from[i]) f(dims[c->h_ord[from[i]].e1], dims[c->h_ord[from[i]].e2]);
+        if (((classes >> i) & 1) && to[i] > from[i])
+            f(dims[c->h_ord[from[i]].e1], dims[c->h_ord[from[i]].e2], from[i], to[i]);
 }
 
-// Nodes per CTA of the largest class plane under a C-CTA split.
-static int sweep_nloc_max(const shd_ctx *c, int C)
+// Nodes per CTA of the largest of the classes' planes under a C-CTA split.
+static int sweep_nloc_max(const shd_ctx *c, int C, int classes = kAllClasses)
 {
     int m = 0;
-    each_plane(c, [&](int n1, int n2) {
+    each_plane(c, classes, [&](int n1, int n2, int, int) {
         const int R = C == 1 ? n1 : sweep_rows_per_cta(n1, n2, C);
         m = std::max(m, (R < n1 ? R : n1) * n2);
     });
     return m;
 }
 
-// Threads that R rows a thread need, the largest class's.
-static int sweep_threads(const shd_ctx *c, int C, int R)
+// Threads that R rows a thread need, the largest plane's.
+static int sweep_threads(const shd_ctx *c, int C, int classes, int R)
 {
     int m = 0;
-    each_plane(c, [&](int n1, int n2) {
+    each_plane(c, classes, [&](int n1, int n2, int, int) {
         const int rows = C == 1 ? n1 : std::min(sweep_rows_per_cta(n1, n2, C), n1);
         m = std::max(m, (rows + R - 1) / R * n2);
     });
@@ -662,53 +676,88 @@ static int sweep_threads(const shd_ctx *c, int C, int R)
 }
 
 // columns of the widest plane
-static int sweep_columns(const shd_ctx *c)
+static int sweep_columns(const shd_ctx *c, int classes)
 {
     int m = 0;
-    each_plane(c, [&](int, int n2) { m = std::max(m, n2); });
+    each_plane(c, classes, [&](int, int n2, int, int) { m = std::max(m, n2); });
     return m;
 }
 
-// R, V, the thread bound of the kernel, the buffers of schedule (C, NT):
-// strides at compile time for R <= 4 where they fit, else at run time; two
-// halo slots only where four leave no plan (planes of some 800 columns and
-// more).  Not built: one row a thread in a cluster (blocks of at most NT nodes
-// run two rows on half the threads) and eight rows below 1024 threads.
-static bool sweep_plan(const shd_ctx *c, SweepSched &sc)
+// The launch of schedule (C, NT) for the classes: R, V, the kernel's thread
+// bound, the buffers.  Strides at compile time for R <= 4 where they fit, else
+// at run time; two halo slots only where four leave no plan (planes of some 600
+// columns and more).  Not built: one row a thread in a cluster (blocks of at
+// most NT nodes run two rows on half the threads) and eight rows below 1024
+// threads.
+static bool sweep_plan(const shd_ctx *c, int C, int NT, int classes, SweepPart &pt)
 {
     const size_t limit = 227 * 1024;
-    const int ps = ((sweep_nloc_max(c, sc.C) + 3) & ~3) + (sc.C == 1 ? 4 : 0);
+    const int ps = ((sweep_nloc_max(c, C, classes) + 3) & ~3) + (C == 1 ? 4 : 0);
     static const int Rs[7] = {1, 2, 3, 4, 6, 8, 1}, Vs[7] = {1, 1, 1, 1, 1, 1, 4};
-    sc.hs = sc.C > 1 ? sweep_columns(c) : 0;
-    for (sc.hsh = kHaloShift; sc.hsh >= (sc.C > 1 ? 1 : kHaloShift); --sc.hsh)
+    pt.hs = C > 1 ? sweep_columns(c, classes) : 0;
+    for (pt.hsh = kHaloShift; pt.hsh >= (C > 1 ? 1 : kHaloShift); --pt.hsh)
         for (int i = 0; i < 7; ++i) {
             const int R = Rs[i], V = Vs[i];
-            if ((R == 8 && sc.NT != 1024) || (R == 1 && V == 1 && sc.C > 1)) continue;
-            const int slots = sweep_threads(c, sc.C, R);
-            if (slots > sc.NT * V) continue;
+            if ((R == 8 && NT != 1024) || (R == 1 && V == 1 && C > 1)) continue;
+            const int slots = sweep_threads(c, C, classes, R);
+            if (slots > NT * V) continue;
             const int nthr = ((slots + V - 1) / V + 31) & ~31;
             // one CTA a plane of 513 to 768 threads: the kernel bounded by 768,
             // with 85 registers a thread instead of 64
-            const int cap = sc.C == 1 && sc.NT == 1024 && V == 1 && R <= 6 && nthr > 512 && nthr <= 768 ? 768 : sc.NT;
-            for (int rt = R > 4 || V > 1 || sc.hsh != kHaloShift; rt < (R > 2 || V > 1 ? 2 : 1); ++rt) {
-                sc.ns = rt ? (slots + 3) & ~3 : cap * V;
-                sc.pstride = rt ? ps : cap * V * R + 8;
-                sc.smem = sizeof(float) * (6 * (size_t)sc.pstride + 2 * (size_t)sc.ns * 3 * R) +
-                          (sc.C > 1 ? ((size_t)1 << sc.hsh) * (16 * (size_t)sc.hs + 16) : 0);
-                if (sc.pstride < ps || sc.smem > limit) continue;
-                sc.R = R;
-                sc.V = V;
-                sc.rt = rt != 0;
-                sc.nthr = nthr;
-                sc.cap = cap;
+            const int cap = C == 1 && NT == 1024 && V == 1 && R <= 6 && nthr > 512 && nthr <= 768 ? 768 : NT;
+            for (int rt = R > 4 || V > 1 || pt.hsh != kHaloShift; rt < (R > 2 || V > 1 ? 2 : 1); ++rt) {
+                pt.ns = rt ? (slots + 3) & ~3 : cap * V;
+                pt.pstride = rt ? ps : cap * V * R + 8;
+                pt.smem = sizeof(float) * (6 * (size_t)pt.pstride + 2 * (size_t)pt.ns * 3 * R) +
+                          (C > 1 ? ((size_t)1 << pt.hsh) * (16 * (size_t)pt.hs + 16) : 0);
+                if (pt.pstride < ps || pt.smem > limit) continue;
+                pt.R = R;
+                pt.V = V;
+                pt.rt = rt != 0;
+                pt.nthr = nthr;
+                pt.cap = cap;
+                pt.k0 = c->N;
+                pt.k1 = 0;
+                each_plane(c, classes, [&](int, int, int k0, int k1) {
+                    pt.k0 = std::min(pt.k0, k0);
+                    pt.k1 = std::max(pt.k1, k1);
+                });
                 return true;
             }
         }
     return false;
 }
 
+// The launches of (C, NT); false where a plane finds no plan (none of the
+// schedules sweep_sched_make accepts).
+static bool sweep_parts(const shd_ctx *c, SweepSched &sc)
+{
+    SweepPart all;
+    if (!sweep_plan(c, sc.C, sc.NT, kAllClasses, all)) return false;
+    sc.part[0] = all;
+    sc.nparts = 1;
+    if (!all.rt) return true;
+    int mask[3], n = 0;  // runs of classes of one R and V
+    SweepPart pt, last;
+    for (int i = 0; i < 3; ++i) {
+        bool present = false;
+        each_plane(c, 1 << i, [&](int, int, int, int) { present = true; });
+        if (!present || !sweep_plan(c, sc.C, sc.NT, 1 << i, pt)) continue;
+        if (n > 0 && pt.R == last.R && pt.V == last.V) mask[n - 1] |= 1 << i;
+        else mask[n++] = 1 << i;
+        last = pt;
+    }
+    for (int i = 0; i < n; ++i)
+        if (!sweep_plan(c, sc.C, sc.NT, mask[i], sc.part[i])) {
+            sc.part[0] = all;
+            return true;
+        }
+    sc.nparts = n;
+    return true;
+}
+
 using SweepKernel = void (*)(Prob<float>, float *, const float *, const float *, const float *,
-                             const unsigned long long *, int, int, int, int, int, int, int, int *, int);
+                             const unsigned long long *, int, int, int, int, int, int, int, int *, int, int);
 
 template <int R, int V, int NT, int NS, bool CL>
 static SweepKernel sweep_kernel_of()
@@ -730,7 +779,7 @@ static SweepKernel sweep_kernel_ns(int R)
 }
 
 template <bool CL>
-static SweepKernel sweep_kernel(const SweepSched &sc)
+static SweepKernel sweep_kernel(const SweepPart &sc)
 {
     if (sc.rt) {  // one instantiation for every thread count up to 1024 (64 registers)
         if (sc.V == 4) return sc.R == 1 ? sweep_kernel_of<1, 4, 1024, 0, CL>() : nullptr;
@@ -752,43 +801,53 @@ static SweepKernel sweep_kernel(const SweepSched &sc)
     return nullptr;
 }
 
-// Run schedule sc over `n` (ordinate, group) pairs (all of them, or every
-// tune_stride-th into a scratch intensity when timing).
+// Run schedule sc over every (ordinate, group) pair or, when timing, over the
+// first n of every tune_stride-th into a scratch intensity.
 static cudaError_t run_sweep_sched(const shd_ctx *ctx, const SweepSched &sc, float *I, const float *eta,
                                    const float *chi, cudaStream_t st, bool bits, bool wide, int n, int tune_stride)
 {
     Prob<float> P = make_prob<float>(ctx);
     const float *c0L = bits ? (const float *)ctx->d_chi0L : nullptr;
     const unsigned long long *mb = bits ? ctx->d_mbits : nullptr;
-    SweepKernel kern = sc.C > 1 ? sweep_kernel<true>(sc) : sweep_kernel<false>(sc);
-    if (!kern) return cudaErrorInvalidConfiguration;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sc.smem);
-    if (e != cudaSuccess) return e;
-    // the whole unified L1 as shared memory, so that the CTAs the register
-    // budget allows also fit there
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    if (e != cudaSuccess) return e;
-    if (sc.C > 8) {  // 16-CTA clusters are beyond the portable size: opted in per kernel
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    for (int i = 0; i < sc.nparts; ++i) {
+        const SweepPart &pt = sc.part[i];
+        int first = pt.k0 * ctx->G, end = pt.k1 * ctx->G;
+        if (tune_stride > 0) {
+            first = (first + tune_stride - 1) / tune_stride;
+            end = std::min(n, (end + tune_stride - 1) / tune_stride);
+        }
+        if (end <= first) continue;
+        SweepKernel kern = sc.C > 1 ? sweep_kernel<true>(pt) : sweep_kernel<false>(pt);
+        if (!kern) return cudaErrorInvalidConfiguration;
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pt.smem);
         if (e != cudaSuccess) return e;
+        // the whole unified L1 as shared memory, so that the CTAs the register
+        // budget allows also fit there
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        if (e != cudaSuccess) return e;
+        if (sc.C > 8) {  // 16-CTA clusters are beyond the portable size: opted in per kernel
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            if (e != cudaSuccess) return e;
+        }
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)((end - first) * sc.C));
+        cfg.blockDim = dim3((unsigned)pt.nthr);
+        cfg.dynamicSmemBytes = pt.smem;
+        cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)sc.C;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = sc.C > 1 ? 1 : 0;
+        e = cudaLaunchKernelEx(&cfg, kern, P, I, eta, chi, c0L, mb, ctx->mbits_npc, ctx->mbits_nwin, pt.pstride, pt.ns,
+                               pt.hs, pt.hsh, wide ? 1 : 0, ctx->d_tc_err, first, tune_stride);
+        note_launch();
+        if (e != cudaSuccess) return e;
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(n * sc.C));
-    cfg.blockDim = dim3((unsigned)sc.nthr);
-    cfg.dynamicSmemBytes = sc.smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)sc.C;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = sc.C > 1 ? 1 : 0;
-    e = cudaLaunchKernelEx(&cfg, kern, P, I, eta, chi, c0L, mb, ctx->mbits_npc, ctx->mbits_nwin, sc.pstride, sc.ns, sc.hs,
-                           sc.hsh, wide ? 1 : 0, ctx->d_tc_err, tune_stride);
-    note_launch();
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
 // The schedule (C, NT) is one of this problem's: planes of at most 4 NT nodes
@@ -814,7 +873,7 @@ static bool sweep_sched_make(const shd_ctx *c, int C, int NT, SweepSched &sc)
     }
     sc.C = C;
     sc.NT = NT;
-    return sweep_plan(c, sc);  // (every schedule of these bounds has one)
+    return sweep_parts(c, sc);  // (every schedule of these bounds has its plans)
 }
 
 // Every schedule that fits, one CTA a plane first.
@@ -915,15 +974,18 @@ static bool sweep_schedule(const shd_ctx *cc, cudaStream_t st, const float *eta,
 // two rows under the 64 registers of 1024 threads spill without a launch's
 // constant operands (three 64^3 jets 23.6 ms, 19.3 in launches of their own,
 // 22.5 before; 52^3 19.3, 15.8, 17.9): those problems sweep on their own.
-static bool sweep_batch_plan(const shd_ctx *c, SweepSched &sc)
+static bool sweep_batch_plan(const shd_ctx *c, SweepPart &pt)
 {
-    return sweep_sched_make(c, 1, 1024, sc) && sc.V == 1 && !sc.rt && (sc.R <= 2 || sc.cap == 768);
+    SweepSched sc;
+    if (!sweep_sched_make(c, 1, 1024, sc) || sc.nparts != 1) return false;
+    pt = sc.part[0];
+    return pt.V == 1 && !pt.rt && (pt.R <= 2 || pt.cap == 768);
 }
 
 size_t sweep_batch_smem(const shd_ctx *c)
 {
-    SweepSched sc;
-    return sweep_batch_plan(c, sc) ? sc.smem : 0;
+    SweepPart pt;
+    return sweep_batch_plan(c, pt) ? pt.smem : 0;
 }
 
 // the descriptor of problem c as its own sweep launch would see it
@@ -939,18 +1001,18 @@ void sweep_batch_fill(const shd_ctx *c, SweepBatchProb &d, long long item0)
     d.npc = c->mbits_npc;
     d.nwin = c->mbits_nwin;
     d.wide = sweep_tau_bounded(c) ? 0 : 1;
-    SweepSched sc;
-    sweep_batch_plan(c, sc);
-    d.pstride = sc.pstride;
-    d.ns = sc.ns;
+    SweepPart pt;
+    sweep_batch_plan(c, pt);
+    d.pstride = pt.pstride;
+    d.ns = pt.ns;
     d.item0 = item0;
 }
 
 int sweep_batch_class(const shd_ctx *c)
 {
     if (c->precision == SHD_FP64 || c->integrator != SHD_SC_LINEAR) return 0;
-    SweepSched sc;
-    if (!sweep_batch_plan(c, sc)) return 0;
+    SweepPart pt;
+    if (!sweep_batch_plan(c, pt)) return 0;
     if (c->sweep_force_C > 0 && !(c->sweep_force_C == 1 && c->sweep_force_NT == 1024)) return 0;
     if (c->sweep_force_C <= 0 && c->sweep_C > 0 && !(c->sweep_C == 1 && c->sweep_NT == 1024)) {
         // another schedule won the problem's timing: it joins only if the
@@ -962,7 +1024,7 @@ int sweep_batch_class(const shd_ctx *c)
         }
         if (!(pp > 0.f && pp <= 1.03f * best)) return 0;
     }
-    return sc.R * 8 + sc.cap / 256;
+    return pt.R * 8 + pt.cap / 256;
 }
 
 cudaError_t launch_sweep_batch(int cls, const SweepBatchProb *d_probs, int nprob, long long nitems, size_t smem,
