@@ -576,9 +576,8 @@ __device__ inline float fast_recip<float>(float x) { return hw_rcp(x); }
 // only for the 4-node pieces of a plane that hold a moving node (bit id % 64
 // of mbits[d][id / 64][piece]) and from chi0L elsewhere; the CTA keeps the
 // current 64-plane window of its layout's bits in shared memory.
-// WIDE (single precision): the weights' exponential carries the remainder of
-// its argument (exp_neg); launched unless the host bound excludes optical
-// depths above kTauPlain.
+// WIDE (single precision): steps beyond kTauPlain take sc_weights_above;
+// launched unless the host bound excludes such depths.
 template <class T, int U, bool VEC, bool CB, bool WIDE>
 __global__ void __launch_bounds__(1024, 1) k_sweep_pipe(Prob<T> P, T *__restrict__ I, const T *__restrict__ eta,
                                                         const T *__restrict__ chi, const T *__restrict__ chi0L,
@@ -883,8 +882,8 @@ __global__ void __launch_bounds__(1024, 1) k_sweep_bez(Prob<T> P, T *__restrict_
                         dP = (x > T(0) && xd > T(0))
                                  ? fb_derivative<T>(slope, bounded_slope<T>(quot<T>(sD - sP, xd)), x, xd)
                                  : T(0);
-                    const T Cu = clamp_between<T>(su + x * du * T(1.0 / 3.0), su, sP);
-                    const T Cp = clamp_between<T>(sP - x * dP * T(1.0 / 3.0), su, sP);
+                    const T Cu = clamp_between<T>(su + third<T>(x * du), su, sP);
+                    const T Cp = clamp_between<T>(sP - third<T>(x * dP), su, sP);
                     T e, wU, wCU, wCP, wP;
                     bezier_weights<T>(x, e, wU, wCU, wCP, wP);
                     inew = iu * e + wU * su + wCU * Cu + wCP * Cp + wP * sP;
@@ -1751,7 +1750,7 @@ static cudaError_t launch_sweep_pipe(const shd_ctx *ctx, T *I, const T *eta, con
     const T *c0L = bits ? (const T *)ctx->d_chi0L : nullptr;
     const unsigned long long *mb = bits ? ctx->d_mbits : nullptr;
     if (bits) sm += sizeof(unsigned long long) * (size_t)ctx->mbits_npc;
-    // the compensated exponential is needed only if a step's optical depth can exceed kTauPlain
+    // (needed only if a step's optical depth can exceed kTauPlain)
     const bool wide = sizeof(T) == 4 && !sweep_tau_bounded(ctx);
     auto kern = bits ? (wide ? k_sweep_pipe<T, U, VEC, VEC, (sizeof(T) == 4)> : k_sweep_pipe<T, U, VEC, VEC, false>)
                      : (wide ? k_sweep_pipe<T, U, VEC, false, (sizeof(T) == 4)> : k_sweep_pipe<T, U, VEC, false, false>);

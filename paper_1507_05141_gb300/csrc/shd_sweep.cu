@@ -430,18 +430,20 @@ __device__ __forceinline__ void sweep_pair_rays(const Prob<float> &P, const Swee
 #pragma unroll
                 for (int q = 0; q < R; ++q) u[q].x = bc_iso;
             } else {
-                float xm = 1e30f;
+                float xm = 1e30f, xM = 0.f;
 #pragma unroll
                 for (int q = 0; q < R; ++q) {
                     x[q] = hs * (x[q] + ct[q]);
                     xm = fminf(xm, x[q]);
+                    xM = fmaxf(xM, x[q]);
                 }
-                if (xm >= 0.5f) {
+                if (xm >= 0.5f && xM <= kTauPlain) {
                     // every row above the weights' series (a time step's
-                    // kappa s is at least 2 at c dt = half a node spacing)
+                    // kappa s is at least 2 at c dt = half a node spacing) and
+                    // within the plain exponential
 #pragma unroll
                     for (int q = 0; q < R; ++q) {
-                        const float e = wide ? exp_neg(x[q]) : hw_exp2(-x[q] * kLog2eF);
+                        const float e = hw_exp2(-x[q] * kLog2eF);
                         const float a0 = (1.f - e) * hw_rcp(x[q]);
                         u[q].x = fmaf(u[q].y, a0 - e, fmaf(st[q], 1.f - a0, u[q].x * e));
                     }
