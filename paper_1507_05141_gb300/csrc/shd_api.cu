@@ -777,9 +777,6 @@ int ready_for_step(shd_ctx *c)
     if (remap_smem_bytes(c) > limit)
         return fail(SHD_ERR_ARG, "groups x ordinates too large for the remap kernels (%zu bytes shared memory)",
                     remap_smem_bytes(c));
-    if (sh2lab_tile_smem_bytes(c) > limit)
-        return fail(SHD_ERR_ARG, "too many harmonics for the sh2lab kernel (%zu bytes shared memory)",
-                    sh2lab_tile_smem_bytes(c));
     if (sweep_smem_bytes(c) > limit) return fail(SHD_ERR_ARG, "grid planes too large for the sweep kernel");
     if (c->integrator == SHD_SC_BEZIER && !sweep_bez_usable(c))
         return fail(SHD_ERR_ARG, "grid planes too large for the Bezier sweep (at most 4096 nodes, %zu bytes "

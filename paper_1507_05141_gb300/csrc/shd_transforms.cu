@@ -162,97 +162,6 @@ __global__ void __launch_bounds__(128) k_sh2lab_f64(Prob<double> P, const double
 }
 
 // -------------------------------------------------------------------------
-// a3: [64 x NLM] x [NLM x N] per (tile, group), N in chunks of 128
-// ordinates; 256 threads = 8 row groups of 8 rows x 32 column groups of 4.
-// -------------------------------------------------------------------------
-template <class T>
-__global__ void __launch_bounds__(256) k_sh2lab_tile(Prob<T> P, const T *__restrict__ Sp, T *__restrict__ eta,
-                                                     T *__restrict__ chi, T *__restrict__ S0)
-{
-    constexpr int R = 64, KC = 128, TR = 8, TC = 4;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int NLM = P.NLM;
-    T *As = reinterpret_cast<T *>(smem_raw);  // [NLM][R]
-    T *Bs = As + (size_t)NLM * R;             // [NLM][KC]
-    T *Cs = Bs + (size_t)NLM * KC;            // [KC][R + 1]
-    T *chir = Cs + (size_t)KC * (R + 1);      // [R]
-    int *mrow = reinterpret_cast<int *>(chir + R);  // [R] moving index of the row, -1 at rest
-    const int tile = blockIdx.x / P.G, g = blockIdx.x - (blockIdx.x / P.G) * P.G;
-    const TileInfo ti = P.tiles[tile];
-    const int tid = threadIdx.x, tr = tid >> 5, tc = tid & 31;
-
-    for (int e = tid; e < R * NLM; e += 256) {
-        int r = e / NLM, p = e - r * NLM;
-        int ix = ti.x0 + (r & 7), iy = ti.y0 + (r >> 3);
-        T v = T(0);
-        if (ix < P.nx && iy < P.ny) {
-            long long c = ((long long)ti.z * P.ny + iy) * P.nx + ix;
-            v = Sp[(c * P.G + g) * NLM + p];
-        }
-        As[(size_t)p * R + r] = v;
-    }
-    for (int r = tid; r < R; r += 256) {
-        int ix = ti.x0 + (r & 7), iy = ti.y0 + (r >> 3);
-        T ch = T(0);
-        int m = -1;
-        if (ix < P.nx && iy < P.ny) {
-            long long c = ((long long)ti.z * P.ny + iy) * P.nx + ix;
-            ch = P.chi0[c * P.G + g];
-            m = P.midx[c];
-        }
-        chir[r] = ch;
-        mrow[r] = m;
-    }
-    for (int k0 = 0; k0 < P.N; k0 += KC) {
-        for (int e = tid; e < KC * NLM; e += 256) {
-            int kk = e / NLM, p = e - kk * NLM, k = k0 + kk;
-            Bs[(size_t)p * KC + kk] = k < P.N ? P.Y[(size_t)k * NLM + p] : T(0);
-        }
-        __syncthreads();
-        T acc[TR][TC];
-#pragma unroll
-        for (int i = 0; i < TR; ++i)
-#pragma unroll
-            for (int j = 0; j < TC; ++j) acc[i][j] = T(0);
-        for (int p = 0; p < NLM; ++p) {
-            T a[TR], b[TC];
-#pragma unroll
-            for (int i = 0; i < TR; ++i) a[i] = As[(size_t)p * R + tr * TR + i];
-#pragma unroll
-            for (int j = 0; j < TC; ++j) b[j] = Bs[(size_t)p * KC + tc + 32 * j];
-#pragma unroll
-            for (int i = 0; i < TR; ++i)
-#pragma unroll
-                for (int j = 0; j < TC; ++j) acc[i][j] += a[i] * b[j];
-        }
-#pragma unroll
-        for (int i = 0; i < TR; ++i)
-#pragma unroll
-            for (int j = 0; j < TC; ++j) Cs[(size_t)(tc + 32 * j) * (R + 1) + tr * TR + i] = acc[i][j];
-        __syncthreads();
-        for (int e = tid; e < KC * R; e += 256) {
-            int kk = e >> 6, q = e & 63, k = k0 + kk;
-            if (k >= P.N) continue;
-            int d = P.ord[k].d;
-            int r = tile_row(d, q);
-            int ix = ti.x0 + (r & 7), iy = ti.y0 + (r >> 3);
-            if (ix >= P.nx || iy >= P.ny) continue;
-            T v = Cs[(size_t)kk * (R + 1) + r];
-            const int m = mrow[r];
-            if (m >= 0) {
-                S0[((long long)m * P.G + g) * P.N + k] = v;  // comoving, node-major
-            } else {
-                long long a = ((long long)k * P.G + g) * P.Nc + perm_offset(d, ix, iy, ti.z, P.nx, P.ny, P.nz);
-                T ch = chir[r];
-                eta[a] = ch * v;
-                chi[a] = ch;
-            }
-        }
-        __syncthreads();
-    }
-}
-
-// -------------------------------------------------------------------------
 // Single precision.  Both contractions are bound by the FP32 FMA rate (about
 // 65 TFLOP/s reachable; 2 x 65.5 kflop per node and group at L = 7), so the
 // tiles are chosen for FMAs per shared-memory load: 16 x TN (a1) and 4 x 16
@@ -1580,19 +1489,12 @@ __global__ void __launch_bounds__(512, 2) k_moments_f32(Prob<float> P, const flo
     }
 }
 
-size_t sh2lab_tile_smem_bytes(const shd_ctx *c)
-{
-    return (size_t)c->esize * ((size_t)c->NLM * 64 + (size_t)c->NLM * 128 + 128 * 65 + 64) + 64 * 4 + 64;
-}
-
 static int num_sms(const shd_ctx *ctx)
 {
     int n = 0;
     if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess || n <= 0) n = 148;
     return n;
 }
-
-static const size_t kSmemLimit = 227 * 1024;
 
 // rows of the grid along x and y are 16-byte multiples
 static bool rows_aligned(const shd_ctx *c) { return c->nx % 4 == 0 && c->ny % 4 == 0; }
@@ -1625,7 +1527,6 @@ static cudaError_t launch_project_f32_tn(const shd_ctx *ctx, int tn, const float
         case 5: return launch_project_f32_k<5, ROWS, VEC>(ctx, I, Ip, mom, nmo, st);
         case 6: return launch_project_f32_k<6, ROWS, VEC>(ctx, I, Ip, mom, nmo, st);
         case 7: return launch_project_f32_k<7, ROWS, VEC>(ctx, I, Ip, mom, nmo, st);
-        case 8: return launch_project_f32_k<8, ROWS, VEC>(ctx, I, Ip, mom, nmo, st);
         default: return cudaErrorInvalidConfiguration;
     }
 }
@@ -1650,11 +1551,9 @@ static size_t sh2lab_f32_smem_bytes(const shd_ctx *c)
                             (size_t)2 * 64 * ((c->NLM + 31) & ~31) + 256);
 }
 
-// FP32's a3 keeps chi_lab at rest (as the mixed segment transform does)
-bool sh2lab_f32_usable(const shd_ctx *c)
-{
-    return c->precision == SHD_FP32 && sh2lab_f32_smem_bytes(c) <= kSmemLimit;
-}
+// FP32's a3 keeps chi_lab at rest (as the mixed segment transform does); its
+// slices fit every order (124 KB at L = 9)
+bool sh2lab_f32_usable(const shd_ctx *c) { return c->precision == SHD_FP32; }
 
 template <int ROWS>
 static cudaError_t launch_sh2lab_f32_k(const shd_ctx *ctx, const float *Sp, float *eta, float *chi, float *S0,
@@ -1824,32 +1723,18 @@ cudaError_t launch_sh2lab(const shd_ctx *ctx, const T *Sp, T *eta, T *chi, cudaS
     Prob<T> P = make_prob<T>(ctx);
     cudaError_t e = cudaSuccess;
     T *nm0 = (T *)ctx->d_nm[0], *nm1 = (T *)ctx->d_nm[1], *nm2 = (T *)ctx->d_nm[2];
-    bool done = false;
     if constexpr (sizeof(T) == 4) {
         // the segment kernels run the remap and write the moving rows themselves
         if (seg_usable(ctx)) return launch_sh2lab_seg(ctx, Sp, eta, chi, nm0, nm1, nm2, st, full_chi);
-        if (tc_usable(ctx)) {
-            if ((e = launch_sh2lab_tc(ctx, Sp, eta, chi, nm0, st)) != cudaSuccess) return e;
-            done = true;
-        } else if (sh2lab_f32_smem_bytes(ctx) <= kSmemLimit) {
-            if ((e = launch_sh2lab_f32(ctx, Sp, eta, chi, nm0, st, full_chi || !sh2lab_f32_usable(ctx))) != cudaSuccess)
-                return e;
-            done = true;
-        }
-    }
-    if constexpr (sizeof(T) == 8) {
+        e = tc_usable(ctx) ? launch_sh2lab_tc(ctx, Sp, eta, chi, nm0, st)
+                           : launch_sh2lab_f32(ctx, Sp, eta, chi, nm0, st, full_chi || !sh2lab_f32_usable(ctx));
+        if (e != cudaSuccess) return e;
+    } else {
         const int nsl = (ctx->N + 7) / 8;
         const size_t sm = sizeof(double) * 65 * (size_t)ctx->NLM;
         e = cudaFuncSetAttribute(k_sh2lab_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
         k_sh2lab_f64<<<(unsigned)(ctx->ntiles * ctx->G * nsl), 128, sm, st>>>(P, Sp, eta, chi, nm0, nsl);
-        note_launch();
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    } else if (!done) {
-        size_t sm = sh2lab_tile_smem_bytes(ctx);
-        e = cudaFuncSetAttribute(k_sh2lab_tile<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-        k_sh2lab_tile<T><<<(unsigned)(ctx->ntiles * ctx->G), 256, sm, st>>>(P, Sp, eta, chi, nm0);
         note_launch();
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
