@@ -1459,7 +1459,28 @@ __global__ void __launch_bounds__(256) k_source_thermal(Prob<T> P, const T *__re
 // layout conversions
 // -------------------------------------------------------------------------
 // Canonical FP64 [c][g][k] (mesh order) <-> the discrete-ordinate layout
-// [k][g][o], TO_DO or back: an 8 x 8 brick of nodes in one group per CTA, 32
+// [k][g][o], TO_DO or back.  Small states: a thread an element, the canonical
+// side contiguous; the other moves 4 bytes of a 32-byte sector, which L2 holds
+// until its neighbours come.
+template <class T, bool TO_DO>
+__global__ void __launch_bounds__(256) k_state_elements(Prob<T> P, const double *__restrict__ canon_in,
+                                                        double *__restrict__ canon_out, T *__restrict__ dov,
+                                                        long long c0, long long n)
+{
+    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int k = (int)(i % P.N);
+    const long long cg = i / P.N;
+    const int g = (int)(cg % P.G);
+    int ix, iy, iz;
+    node_xyz(c0 + cg / P.G, P.nx, P.ny, ix, iy, iz);
+    const int ki = P.mesh2int[k];
+    const long long a = ((long long)ki * P.G + g) * P.Nc + perm_offset(P.ord[ki].d, ix, iy, iz, P.nx, P.ny, P.nz);
+    if constexpr (TO_DO) dov[a] = (T)canon_in[i];
+    else canon_out[i] = (double)dov[a];
+}
+
+// Large states: an 8 x 8 brick of nodes in one group per CTA, 32
 // mesh ordinates at a time through shared memory.  The canonical side moves
 // in 256-byte rows of ordinates, the other in 32-byte runs of nodes; a
 // thread's eight values of a chunk are in flight together.  One thread an
@@ -2061,12 +2082,28 @@ static cudaError_t launch_state_transpose(const shd_ctx *ctx, const double *in, 
                                           long long nc, cudaStream_t st)
 {
     if (nc * ctx->G * ctx->N == 0) return cudaSuccess;
-    const long long layer = (long long)ctx->nx * ctx->ny;
+    const long long layer = (long long)ctx->nx * ctx->ny, n = nc * ctx->G * ctx->N;
+    const long long tiles = (long long)((ctx->nx + 7) / 8) * ((ctx->ny + 7) / 8);
+    // an element a thread where L2 holds the state and the nodes are few or
+    // the bricks would not be full: set, get in FP32 of 16^3, 8 groups, 512
+    // ordinates 127, 114 us, by bricks 139, 137; 4 x 48 x 48, 6 groups 218, 190
+    // (314, 266); 4 x 96 x 96 921, 878 (1377, 1234).  24^3, 4 groups, 128
+    // ordinates by bricks 50, 50 (55, 55); 8 groups, 288 ordinates 196, 171
+    // (241, 215); 32^3, 16 groups 960, 793 (2041, 1966).  33 x 31 x 30, 4 groups,
+    // 128 ordinates 118, 110 (132, 116)
+    const double full = (double)layer / (64.0 * (double)tiles);
+    if (full >= 0.7 ? n <= 20000000 && (nc <= 6000 || full < 0.82) : n <= (full >= 0.6 ? 40000000 : 120000000)) {
+        k_state_elements<T, TO_DO><<<blocks_for(n, 256), 256, 0, st>>>(make_prob<T>(ctx), in, out, dov, c0, n);
+        note_launch();
+        return cudaGetLastError();
+    }
     const int z0 = (int)(c0 / layer), z1 = (int)((c0 + nc - 1) / layer);
-    const long long nbr = (long long)((ctx->nx + 7) / 8) * ((ctx->ny + 7) / 8) * (z1 - z0 + 1);
-    // few bricks: their chunks of ordinates to several CTAs (about eight an SM)
+    const long long nbr = tiles * (z1 - z0 + 1);
+    // few bricks: their chunks of ordinates to several CTAs (about eight waves
+    // of eight an SM: 24^3, 8 groups, 512 ordinates 381 us a set with one wave,
+    // 337 with eight, 368 with a CTA a chunk)
     const int nch = (ctx->N + 31) / 32;
-    const int ny = (int)std::min<long long>(nch, std::max<long long>(1, 1216 / (nbr * ctx->G)));
+    const int ny = (int)std::min<long long>(nch, std::max<long long>(1, 9728 / (nbr * ctx->G)));
     k_state_transpose<T, TO_DO><<<dim3((unsigned)(nbr * ctx->G), (unsigned)ny), 256, 0, st>>>(make_prob<T>(ctx), in, out, dov,
                                                                                            c0, nc, z0, nbr);
     note_launch();
