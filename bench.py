@@ -67,10 +67,9 @@ def sweep_traffic(prec, spec):
                 fields[k.strip()] = v.strip().strip("`")
     csrc = os.path.join(ROOT, "paper_1507_05141_gb300", "csrc")
     try:
-        if fields.get("shd_kernels.cu sha256") != _sha256(os.path.join(csrc, "shd_kernels.cu")):
-            return None
-        if fields.get("shd_internal.cuh sha256") != _sha256(os.path.join(csrc, "shd_internal.cuh")):
-            return None
+        for src in ("shd_sweep.cu", "shd_internal.cuh"):  # the sweep kernels and their weights
+            if fields.get(f"{src} sha256") != _sha256(os.path.join(csrc, src)):
+                return None
         return int(fields["dram bytes per launch"])
     except (KeyError, ValueError, OSError):
         return None
