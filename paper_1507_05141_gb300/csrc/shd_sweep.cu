@@ -50,7 +50,7 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
 // parities (97 instructions an update in the node-a-thread layout, 66 here).
 // NS = 0 takes the strides at run time (rows that do not divide the threads,
 // at the least shared memory).  64^3, 16 groups, 512 ordinates: 8.08 ms a
-// sweep before, 6.05 now, 5.1 TB/s of DRAM traffic, 0.75 of the copy rate.
+// sweep before, 5.9 now, 5.5 TB/s of DRAM traffic, 0.81 of the copy rate.
 //
 // In a cluster the halo row of a CTA's first row block is the last row of
 // the upwind CTA, which sends it: each thread of its last row block writes
@@ -59,7 +59,7 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
 // wait for it.  A slot is handed back by a remote arrive two planes later,
 // so the CTAs of a cluster run as a pipeline a plane or so apart and no
 // plane pays a cluster barrier, its release fence and its wait (128^3, 3
-// groups: 15.5 ms a sweep with a barrier a plane, 14.0 now, with chi at rest
+// groups: 15.5 ms a sweep with a barrier a plane, 14.4 now, with chi at rest
 // from the table; the two CTAs an SM need 106.6 KB each, so the exchange
 // holds no separate halo rows).
 // Waits are bounded: on timeout the thread raises *err and runs on.
